@@ -24,6 +24,7 @@ static void free_system(fv_system* s) {
   free_krylov(s->kry);
   free_batch(s->batch);
   for (void* p : s->allocs) cudaFree(p);
+  if (s->subs.st.err) cudaFreeHost(s->subs.st.err);
   delete s;
 }
 

@@ -400,6 +400,10 @@ static fv_status setup_g(const fv_system* s, BatchWork* bw, size_t tab) {
 
 static fv_status ras_batch(const fv_system* s, BatchWork* bw, int nrhs, const double* r, long long rs, double* z,
                            long long zs, cudaStream_t st) {
+  if (s->subs.st.on) {
+    ProfScope ps(s->kind == FV_VTBE ? FV_K_RAS_FWD_VTBE : FV_K_RAS_FWD_PPBE, st);
+    return ras_stream64(s, nrhs, r, rs, z, zs, bw->loc, st);
+  }
   if (s->d == 2)
     return s->subs.fp32 ? ras_batch_g<float, 2>(s, bw, nrhs, r, rs, z, zs, st)
                         : ras_batch_g<double, 2>(s, bw, nrhs, r, rs, z, zs, st);
@@ -523,16 +527,21 @@ static fv_status ensure_batch(const fv_system* s, int nrhs, int m) {
   const size_t n = (size_t)s->n, R = (size_t)nrhs;
   const size_t gsz = (size_t)s->d * 6 * 4 * s->grid->h.Nr * (s->grid->h.Ns + 2);
   const size_t es = s->subs.fp32 ? 4 : 8;
+  const long long cells = s->subs.st.on ? s->subs.st.sT : s->subs.total_cells;
   if (cudaMalloc(&bw->gh, gsz * R * 8) || cudaMalloc(&bw->V, (m + 1) * n * R * 8) || cudaMalloc(&bw->Z, m * n * R * 8) ||
       cudaMalloc(&bw->w, n * R * 8) || cudaMalloc(&bw->r, n * R * 8) || cudaMalloc(&bw->part, R * BK * BBLOCKS * 8) ||
       cudaMalloc(&bw->h, R * 3 * BK * 8) || cudaMalloc(&bw->coef, R * BK * 8) || cudaMalloc(&bw->ticket, R * 4) ||
-      cudaMalloc(&bw->loc, (size_t)s->subs.total_cells * s->d * R * es) || cudaMalloc(&bw->task, 2 * sizeof(int)) ||
+      cudaMalloc(&bw->loc, (size_t)cells * s->d * R * es) || cudaMalloc(&bw->task, 2 * sizeof(int)) ||
       cudaMallocHost(&bw->hhost, R * 3 * BK * 8) || cudaMallocHost(&bw->coef_host, R * BK * 8) ||
       cudaMalloc(&bw->arn, R * sizeof(BatchArn)) || cudaMallocHost(&bw->arn_host, R * sizeof(BatchArn)) ||
       cudaMemset(bw->ticket, 0, R * 4)) {
     free_batch(bw);
     sm->batch = nullptr;
     return set_error("fv_gmres_solve_batch: device allocation failed"), FV_ENOMEM;
+  }
+  if (s->subs.st.on) {
+    FV_CUDA(cudaMemset(bw->loc, 0, (size_t)cells * s->d * R * es));  // padding cells are copied, never used
+    return FV_OK;
   }
   // autotune the right-hand-side group G of the RAS sweeps on this system and batch size
   const size_t tab = batch_tables_bytes(s);
@@ -743,6 +752,7 @@ fv_status gmres_batch(const fv_system* s, int nrhs, const double* B, double* X, 
     }
     if ((rc = fetch_state())) return rc;
   }
+  if (sweep_failed(s)) return set_error("fv_gmres_solve_batch: a wait of the subdomain sweeps ran out"), FV_ECUDA;
   bool all_conv = true, nan = false;
   for (int t = 0; t < nrhs; ++t) {
     const BatchArn& a = bw->arn_host[t];

@@ -91,6 +91,23 @@ struct fv_grid {
 
 namespace fv {
 
+// operand streams of the fused sweeps (sweep.cu): per component group the box cells in wavefront order, in chunks
+// (a box starts a new chunk) of 16-byte planes of factors and grid cell
+struct SweepStream {
+  int on = 0;                        // 1: the sweeps run from the streams, 0: the general sweeps
+  long long* soff = nullptr;         // [count + 1]
+  long long sT = 0;                  // padded cells
+  unsigned char *fw[2] = {}, *bw[2] = {};
+  int* gather = nullptr;             // [sT] grid cell, -1: none
+  void* loc = nullptr;               // [d][sT] forward results
+  void *shapes = nullptr, *steps = nullptr;  // tables of the distinct box shapes
+  int* shape_of = nullptr;
+  unsigned long long* rows = nullptr;
+  int groups = 0, T = 0, ch_log = 0, loc_smem = 0, table_bytes = 0;  // T: threads of the solve; cells a chunk (log2)
+  size_t smem = 0;
+  int *err = nullptr, *err_dev = nullptr;  // mapped host word: a wait of the sweep ran out
+};
+
 // structured ILU(0) subdomain set of one system on one grid level
 struct Subdomains {
   int count = 0;
@@ -112,7 +129,6 @@ struct Subdomains {
   // order (level i + 2j + k, then j, then i), structure of arrays
   int* perm = nullptr;            // [total_cells] natural local index -> packed position (setup only)
   long long* gmap_p = nullptr;    // [total_cells] packed: global cell or -1
-  int* ijk = nullptr;             // [total_cells] packed: box cell (i | j << 10 | k << 20)
   unsigned char* owned_p = nullptr;
   void* F = nullptr;              // [cell_off * Q + q * ncell + pos], Q = 10 d + d^2, element type per `fp32`
   void* loc = nullptr;            // [cell_off * d + a * ncell + pos] sweep vector
@@ -121,15 +137,9 @@ struct Subdomains {
   int bf16 = 0;                   // 1: factors stored in BF16 (FV_PREC_BF16)
   int max_cols = 0;               // max nx * ny
   int dense_threads = 0;          // CTA size of the level-mapped generic sweeps
-  int dense_single = 0;           // 1: no step is wider than the CTA (the pipelined sweeps apply)
-  size_t smem = 0;                // dynamic shared memory of the sweeps
+  size_t smem = 0;                // dynamic shared memory of the general sweeps
   int ring_in_smem = 0;
-  int stage = 0;                  // d = 2: depth of the shared-memory staged sweeps (8 or 4), 0 = not used
-  size_t stage_off = 0;           // offset of the stage ring in dynamic shared memory
-  int stage_pad = 0;              // zero padding (elements) on each side of the staged sweeps' 4-plane ring
-  size_t stage_smem = 0;          // dynamic shared memory of the staged sweeps
-  void* blk_f = nullptr;          // [total_cells] staged sweeps: forward operand block per packed position
-  void* blk_b = nullptr;          // [total_cells] staged sweeps: backward operand block per packed position
+  SweepStream st;
 };
 
 }  // namespace fv
@@ -232,6 +242,12 @@ fv_status build_subdomains(fv_system* s, const fv_grid* g);
 fv_status ilu_factor(fv_system* s);
 fv_status prepare_sweeps(fv_system* s, int prec);
 fv_status sweeps_smem_attr(const fv_system* s);
+// sweep.cu
+fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::vector<long long>& cell_off, int* used);
+fv_status ras_stream64(const fv_system* s, int nrhs, const double* r, long long rs, double* z, long long zs, void* loc,
+                       cudaStream_t st);
+fv_status ras_stream32(const fv_system* s, const float* r, float* z, cudaStream_t st);
+bool sweep_failed(const fv_system* s);
 fv_status precond_apply(const fv_system* s, const double* r, double* z, cudaStream_t st);
 fv_status precond_apply32(const fv_system* s, const float* r, float* z, cudaStream_t st);
 fv_status ras_apply(const fv_system* s, const double* r, double* z, cudaStream_t st);

@@ -724,6 +724,7 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
     if (!std::isfinite(beta)) nan = true;
     if (breakdown) break;
   }
+  if (sweep_failed(s)) return set_error("fv_gmres_solve: a wait of the subdomain sweeps ran out"), FV_ECUDA;
   const bool conv = !nan && beta <= target;
   if (stats) {
     stats->iters = its;

@@ -342,52 +342,6 @@ __global__ void repack_kernel(int d, int count, const long long* __restrict__ ce
   }
 }
 
-// Per-cell operand blocks of the staged d = 2 sweeps (packed position order, 16-byte multiples so a
-// thread stages its cell's block with 16-byte copies).  Forward: the 5 d lower off-diagonal slots
-// (slot s, component a at s d + a), then L's strictly lower diagonal-block entry (1, 0), then the packed
-// (i, j, k).  Backward: the 5 d upper slots, then U's diagonal block 1 / (0,0), (0,1), 1 / (1,1), the packed
-// (i, j, k) and the scatter target (grid cell of an owned cell, else -1).
-template <class T>
-struct alignas(16) FwdBlk {
-  T f[11];
-  int ijk;
-};
-template <class T>
-struct alignas(16) BwdBlk {
-  T f[13];
-  int ijk;
-  long long go;
-};
-static_assert(sizeof(FwdBlk<float>) == 48 && sizeof(BwdBlk<float>) == 64, "block layout");
-static_assert(sizeof(FwdBlk<double>) == 96 && sizeof(BwdBlk<double>) == 128, "block layout");
-static_assert(sizeof(FwdBlk<__nv_bfloat16>) == 32 && sizeof(BwdBlk<__nv_bfloat16>) == 48, "block layout");
-
-template <class T>
-__global__ void stage_pack_kernel(int count, const long long* __restrict__ cell_off, const T* __restrict__ F,
-                                  const int* __restrict__ ijk, const long long* __restrict__ gmap_p,
-                                  const unsigned char* __restrict__ owned_p, FwdBlk<T>* __restrict__ bf,
-                                  BwdBlk<T>* __restrict__ bb) {
-  constexpr int D = 2, Q = 10 * D + D * D, U = 5 * D + D * D;
-  const long long total = cell_off[count];
-  for (long long C = blockIdx.x * (long long)blockDim.x + threadIdx.x; C < total;
-       C += (long long)gridDim.x * blockDim.x) {
-    const int sd = find_subdomain(cell_off, count, C);
-    const long long base = cell_off[sd], nc = cell_off[sd + 1] - base;
-    const T* Fs = F + base * Q + (C - base);
-    FwdBlk<T> f{};
-    BwdBlk<T> g{};
-    for (int q = 0; q < 5 * D; ++q) f.f[q] = Fs[q * nc], g.f[q] = Fs[(U + q) * nc];
-    f.f[5 * D] = Fs[(5 * D + 1 * D + 0) * nc];
-    g.f[5 * D + 0] = Fs[(5 * D + 0 * D + 0) * nc];
-    g.f[5 * D + 1] = Fs[(5 * D + 0 * D + 1) * nc];
-    g.f[5 * D + 2] = Fs[(5 * D + 1 * D + 1) * nc];
-    f.ijk = g.ijk = ijk[C];
-    g.go = owned_p[C] ? gmap_p[C] : -1;
-    bf[C] = f;
-    bb[C] = g;
-  }
-}
-
 constexpr int DENSE_THREADS = 384;  // CTA size bound of the generic sweeps (170 registers per thread)
 
 static size_t table_bytes(int levels, int ny) { return (size_t)(levels + 1 + levels * ny) * sizeof(int); }
@@ -400,6 +354,33 @@ fv_status prepare_sweeps(fv_system* s, int prec) {
   const size_t es = fp32 ? sizeof(float) : sizeof(double);  // the sweep vectors and rings
   S.fp32 = fp32;
   S.bf16 = prec == 2;
+  // the widest box's level table and wavefront step
+  std::vector<int> dims(3 * S.count);
+  std::vector<long long> cell_off(S.count + 1);
+  FV_CUDA(cudaMemcpy(dims.data(), S.dims, dims.size() * sizeof(int), cudaMemcpyDeviceToHost));
+  FV_CUDA(cudaMemcpy(cell_off.data(), S.cell_off, cell_off.size() * sizeof(long long), cudaMemcpyDeviceToHost));
+  size_t tab = 0;
+  int widest = 1;  // most cells in one wavefront step of any box
+  for (int sd = 0; sd < S.count; ++sd) {
+    const int nx = dims[3 * sd], ny = dims[3 * sd + 1], nz = dims[3 * sd + 2];
+    if (nx >= 1024 || ny >= 1024 || nz >= 1024) return set_error("fv_assemble_system: subdomain too large"), FV_EINVAL;
+    const int levels = (nx - 1) + 2 * (ny - 1) + (nz - 1) + 1;
+    tab = std::max(tab, table_bytes(levels, ny));
+    for (int L = 0; L < levels; ++L) {
+      int cnt = 0;
+      for (int j = 0; j < ny; ++j) cnt += std::max(0, std::min(nx - 1, L - 2 * j) - std::max(0, L - 2 * j - (nz - 1)) + 1);
+      widest = std::max(widest, cnt);
+    }
+  }
+  // boxes whose wavefronts fit a CTA run the streamed sweeps (sweep.cu); wider ones the general sweeps below
+  if (fv_status rc = build_stream(s, dims, cell_off, &S.st.on)) return rc;
+  if (S.st.on) {
+    for (void* p : {(void*)S.off, (void*)S.diag, (void*)S.perm, (void*)S.order, (void*)S.gmap, (void*)S.owned,
+                    (void*)S.gmap_p, (void*)S.owned_p})
+      release(s, p);
+    S.off = S.diag = nullptr, S.perm = S.order = nullptr, S.gmap = S.gmap_p = nullptr, S.owned = S.owned_p = nullptr;
+    return FV_OK;
+  }
   S.F = S.bf16 ? (void*)dalloc<__nv_bfloat16>(s, (size_t)S.total_cells * Q)
         : fp32 ? (void*)dalloc<float>(s, (size_t)S.total_cells * Q)
                : (void*)dalloc<double>(s, (size_t)S.total_cells * Q);
@@ -417,42 +398,7 @@ fv_status prepare_sweeps(fv_system* s, int prec) {
   release(s, S.off), release(s, S.diag), release(s, S.perm);
   S.off = S.diag = nullptr;
   S.perm = nullptr;
-  // the widest box's level table and wavefront step; the 4-plane ring in shared memory when it fits
-  std::vector<int> dims(3 * S.count);
-  FV_CUDA(cudaMemcpy(dims.data(), S.dims, dims.size() * sizeof(int), cudaMemcpyDeviceToHost));
-  size_t tab = 0;
-  int widest = 1;  // most cells in one wavefront step of any box
-  for (int sd = 0; sd < S.count; ++sd) {
-    const int nx = dims[3 * sd], ny = dims[3 * sd + 1], nz = dims[3 * sd + 2];
-    const int levels = (nx - 1) + 2 * (ny - 1) + (nz - 1) + 1;
-    tab = std::max(tab, table_bytes(levels, ny));
-    for (int L = 0; L < levels; ++L) {
-      int cnt = 0;
-      for (int j = 0; j < ny; ++j) cnt += std::max(0, std::min(nx - 1, L - 2 * j) - std::max(0, L - 2 * j - (nz - 1)) + 1);
-      widest = std::max(widest, cnt);
-    }
-  }
   S.dense_threads = std::min(DENSE_THREADS, (widest + 31) / 32 * 32);
-  S.dense_single = widest <= S.dense_threads;  // one cell per thread and step: the pipelined sweeps
-  // (i, j, k) of every packed position (wavefront order: step, then j, then i), so the pipelined
-  // sweeps load a cell's coordinates with its factors instead of searching the step's rows
-  {
-    std::vector<long long> off(S.count + 1);
-    FV_CUDA(cudaMemcpy(off.data(), S.cell_off, off.size() * sizeof(long long), cudaMemcpyDeviceToHost));
-    std::vector<int> ijk(S.total_cells);
-    for (int sd = 0; sd < S.count; ++sd) {
-      const int nx = dims[3 * sd], ny = dims[3 * sd + 1], nz = dims[3 * sd + 2];
-      if (nx >= 1024 || ny >= 1024 || nz >= 1024) return set_error("fv_assemble_system: subdomain too large"), FV_EINVAL;
-      long long pos = off[sd];
-      for (int L = 0; L < nx - 1 + 2 * (ny - 1) + nz; ++L)
-        for (int j = 0; j < ny; ++j)
-          for (int i = std::max(0, L - 2 * j - (nz - 1)); i <= std::min(nx - 1, L - 2 * j); ++i)
-            ijk[pos++] = i | j << 10 | (L - i - 2 * j) << 20;
-    }
-    S.ijk = dalloc<int>(s, S.total_cells);
-    if (!S.ijk) return set_error("fv_assemble_system: allocation of the sweep cell table failed"), FV_ENOMEM;
-    FV_CUDA(cudaMemcpy(S.ijk, ijk.data(), ijk.size() * sizeof(int), cudaMemcpyHostToDevice));
-  }
   const size_t ring = 4 * (size_t)S.max_cols * d * es;
   const size_t ring_al = (ring + 15) / 16 * 16;
   S.ring_in_smem = ring_al + tab <= 200 * 1024;
@@ -461,51 +407,6 @@ fv_status prepare_sweeps(fv_system* s, int prec) {
     S.ring = fp32 ? (void*)dalloc<float>(s, (size_t)S.count * 4 * S.max_cols * d)
                   : (void*)dalloc<double>(s, (size_t)S.count * 4 * S.max_cols * d);
     if (!S.ring) return set_error("fv_assemble_system: allocation of the sweep ring failed"), FV_ENOMEM;
-  }
-  // d = 2 boxes whose steps fit the CTA: the shared-memory staged sweeps, 8, 6 or 4 steps deep when
-  // the stage ring fits beside the 4-plane ring and the tables (per thread and slot: the forward's block,
-  // d right-hand side values and an 8-byte cell map entry, or the backward's block and d values)
-  S.stage = 0;
-  if (d == 2 && S.dense_single && S.ring_in_smem) {
-    const size_t fwd = (S.bf16 ? sizeof(FwdBlk<__nv_bfloat16>) : fp32 ? sizeof(FwdBlk<float>) : sizeof(FwdBlk<double>)) +
-                       d * es + 8;
-    const size_t bwd = (S.bf16 ? sizeof(BwdBlk<__nv_bfloat16>) : fp32 ? sizeof(BwdBlk<float>) : sizeof(BwdBlk<double>)) +
-                       d * es;
-    const size_t per = (size_t)S.dense_threads * std::max(fwd, bwd);
-    int max_nx = 0;
-    for (int sd = 0; sd < S.count; ++sd) max_nx = std::max(max_nx, dims[3 * sd]);
-    S.stage_pad = (max_nx + 1) * d;  // the ring's zero padding on each side (elements)
-    const size_t sring = ((4 * (size_t)S.max_cols * d + 2 * S.stage_pad) * es + 15) / 16 * 16;
-    const size_t off = (sring + tab + 15) / 16 * 16;
-    // at most 200 KB a CTA: a 6-deep ring of 221 KB on the 36 x 36 x 20 fine PPBE boxes ran the forward sweep
-    // 29 % slower than the 4-deep one (too little L1 left beside it)
-    for (int sg : {8, 6, 4})
-      if (off + sg * per <= 200 * 1024) {
-        S.stage = sg, S.stage_off = off, S.stage_smem = off + sg * per;
-        break;
-      }
-    if (S.stage) {
-      if (S.bf16) {
-        using B = __nv_bfloat16;
-        S.blk_f = dalloc<FwdBlk<B>>(s, S.total_cells), S.blk_b = dalloc<BwdBlk<B>>(s, S.total_cells);
-        if (S.blk_f && S.blk_b)
-          stage_pack_kernel<B><<<blocks, 256>>>(S.count, S.cell_off, (const B*)S.F, S.ijk, S.gmap_p, S.owned_p,
-                                                (FwdBlk<B>*)S.blk_f, (BwdBlk<B>*)S.blk_b);
-      } else if (fp32) {
-        S.blk_f = dalloc<FwdBlk<float>>(s, S.total_cells), S.blk_b = dalloc<BwdBlk<float>>(s, S.total_cells);
-        if (S.blk_f && S.blk_b)
-          stage_pack_kernel<float><<<blocks, 256>>>(S.count, S.cell_off, (const float*)S.F, S.ijk, S.gmap_p,
-                                                    S.owned_p, (FwdBlk<float>*)S.blk_f, (BwdBlk<float>*)S.blk_b);
-      } else {
-        S.blk_f = dalloc<FwdBlk<double>>(s, S.total_cells), S.blk_b = dalloc<BwdBlk<double>>(s, S.total_cells);
-        if (S.blk_f && S.blk_b)
-          stage_pack_kernel<double><<<blocks, 256>>>(S.count, S.cell_off, (const double*)S.F, S.ijk, S.gmap_p,
-                                                     S.owned_p, (FwdBlk<double>*)S.blk_f, (BwdBlk<double>*)S.blk_b);
-      }
-      if (!S.blk_f || !S.blk_b) return set_error("fv_assemble_system: allocation of the sweep blocks failed"), FV_ENOMEM;
-      FV_CUDA(cudaGetLastError());
-      FV_CUDA(cudaDeviceSynchronize());
-    }
   }
   return FV_OK;
 }
@@ -740,353 +641,6 @@ __global__ void __launch_bounds__(DENSE_THREADS, 1) ras_bwd_kernel(const long lo
 }
 
 
-// Level-mapped sweeps with every thread holding at most one cell a step (the widest step fits the
-// CTA): the next step's factors and right-hand side are loaded into registers before the barrier
-// (they do not depend on this step's results) and the cell map two steps ahead, so a step's
-// critical path is the barrier, shared-memory ring reads and arithmetic.
-template <class T, int D, class V, class FT = T>
-__global__ void __launch_bounds__(DENSE_THREADS, 1) ras_fwd_pipe_kernel(const long long* __restrict__ cell_off,
-                                                                      const int* __restrict__ dims,
-                                                                      const int* __restrict__ lpt,
-                                                                      const FT* __restrict__ F, T* __restrict__ loc,
-                                                                      T* ring_g, int ring_in_smem, int max_cols,
-                                                                      long long N, const long long* __restrict__ gmap_p,
-                                                                      const int* __restrict__ ijk,
-                                                                      const V* __restrict__ r) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int sd = lpt[blockIdx.x];
-  const SweepBox b = sweep_box(cell_off, dims, sd);
-  const size_t ring_bytes = ring_in_smem ? ((4 * (size_t)max_cols * D * sizeof(T) + 15) / 16 * 16) : 0;
-  T* ring = ring_in_smem ? (T*)smem : ring_g + (size_t)blockIdx.x * 4 * max_cols * D;
-  int* lvl = (int*)(smem + ring_bytes);
-  build_tables(b, lvl, nullptr);
-  constexpr int Q = 10 * D + D * D;
-  const FT* Fb = F + b.base * Q;
-  T* Lb = loc + b.base * D;
-  const long long* gm = gmap_p + b.base;
-  const long long nc = b.nc;
-  const int t = threadIdx.x;
-  auto cnt_of = [&](int L) { return L < b.levels ? lvl[L + 1] - lvl[L] : 0; };
-  long long gn = t < cnt_of(0) ? gm[t] : -1;  // cell map entry of the next fetch
-  T y0[D], fl[5 * D], fd[D * D];
-  int ci = 0, cj = 0, ck = 0;
-  long long cp = -1;
-  const int* cells = ijk + b.base;
-  auto fetch = [&](int L) {
-    cp = -1;
-    if (t >= cnt_of(L)) return;
-    cp = lvl[L] + t;
-    const int c = cells[cp];
-    ci = c & 1023, cj = (c >> 10) & 1023, ck = c >> 20;
-    const long long g = gn;
-#pragma unroll
-    for (int a = 0; a < D; ++a) y0[a] = g >= 0 ? (T)r[a * N + g] : T(0);
-#pragma unroll
-    for (int q = 0; q < 5 * D; ++q) fl[q] = fcvt(Fb[q * nc + cp]);
-#pragma unroll
-    for (int a = 1; a < D; ++a)
-#pragma unroll
-      for (int c = 0; c < a; ++c) fd[a * D + c] = fcvt(Fb[(5 * D + a * D + c) * nc + cp]);
-  };
-  fetch(0);
-  gn = t < cnt_of(1) ? gm[lvl[1] + t] : -1;
-  for (int L = 0; L < b.levels; ++L) {
-    if (cp >= 0) {
-      const int i = ci, j = cj, k = ck, col = j * b.nx + i;
-      T* rp = ring + (size_t)((k & 3) * b.ncols) * D;
-      const T* r0 = ring + (size_t)(((k - 1) & 3) * b.ncols + col) * D;
-      T y[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        y[a] = y0[a];
-        if (k > 0) y[a] -= fl[0 * D + a] * r0[a];
-        if (i > 0 && j > 0) y[a] -= fl[1 * D + a] * rp[(col - b.nx - 1) * D + a];
-        if (j > 0) y[a] -= fl[2 * D + a] * rp[(col - b.nx) * D + a];
-        if (j > 0 && i + 1 < b.nx) y[a] -= fl[3 * D + a] * rp[(col - b.nx + 1) * D + a];
-        if (i > 0) y[a] -= fl[4 * D + a] * rp[(col - 1) * D + a];
-#pragma unroll
-        for (int c = 0; c < a; ++c) y[a] -= fd[a * D + c] * y[c];
-      }
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        rp[col * D + a] = y[a];
-        Lb[a * nc + cp] = y[a];
-      }
-    }
-    fetch(L + 1);
-    if (L + 2 < b.levels) gn = t < cnt_of(L + 2) ? gm[lvl[L + 2] + t] : -1;
-    __syncthreads();
-  }
-}
-
-template <class T, int D, class V, class FT = T>
-__global__ void __launch_bounds__(DENSE_THREADS, 1) ras_bwd_pipe_kernel(const long long* __restrict__ cell_off,
-                                                                      const int* __restrict__ dims,
-                                                                      const int* __restrict__ lpt,
-                                                                      const FT* __restrict__ F, const T* __restrict__ loc,
-                                                                      T* ring_g, int ring_in_smem, int max_cols,
-                                                                      long long N, const long long* __restrict__ gmap_p,
-                                                                      const unsigned char* __restrict__ owned_p,
-                                                                      const int* __restrict__ ijk,
-                                                                      V* __restrict__ z) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int sd = lpt[blockIdx.x];
-  const SweepBox b = sweep_box(cell_off, dims, sd);
-  const size_t ring_bytes = ring_in_smem ? ((4 * (size_t)max_cols * D * sizeof(T) + 15) / 16 * 16) : 0;
-  T* ring = ring_in_smem ? (T*)smem : ring_g + (size_t)blockIdx.x * 4 * max_cols * D;
-  int* lvl = (int*)(smem + ring_bytes);
-  build_tables(b, lvl, nullptr);
-  constexpr int Q = 10 * D + D * D, U = 5 * D + D * D;
-  const int* cells = ijk + b.base;
-  const FT* Fb = F + b.base * Q;
-  const T* Lb = loc + b.base * D;
-  const long long* gm = gmap_p + b.base;
-  const unsigned char* ow = owned_p + b.base;
-  const long long nc = b.nc;
-  const int t = threadIdx.x;
-  T x0[D], fu[5 * D], fd[D * D];
-  int ci = 0, cj = 0, ck = 0;
-  long long cp = -1, go = -1;  // go: cell map entry of an owned cell, else -1
-  auto fetch = [&](int L) {
-    cp = -1;
-    if (L < 0 || t >= lvl[L + 1] - lvl[L]) return;
-    cp = lvl[L] + t;
-    const int c = cells[cp];
-    ci = c & 1023, cj = (c >> 10) & 1023, ck = c >> 20;
-#pragma unroll
-    for (int a = 0; a < D; ++a) x0[a] = Lb[a * nc + cp];
-#pragma unroll
-    for (int q = 0; q < 5 * D; ++q) fu[q] = fcvt(Fb[(U + q) * nc + cp]);
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-      for (int c = a; c < D; ++c) fd[a * D + c] = fcvt(Fb[(5 * D + a * D + c) * nc + cp]);
-    const long long g = gm[cp];
-    go = ow[cp] ? g : -1;
-  };
-  fetch(b.levels - 1);
-  for (int L = b.levels - 1; L >= 0; --L) {
-    if (cp >= 0) {
-      const int i = ci, j = cj, k = ck, col = j * b.nx + i;
-      T* rp = ring + (size_t)((k & 3) * b.ncols) * D;
-      const T* r1 = ring + (size_t)(((k + 1) & 3) * b.ncols + col) * D;
-      T x[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) x[a] = x0[a];
-#pragma unroll
-      for (int a = D - 1; a >= 0; --a) {
-#pragma unroll
-        for (int c = a + 1; c < D; ++c) x[a] -= fd[a * D + c] * x[c];
-        if (i + 1 < b.nx) x[a] -= fu[0 * D + a] * rp[(col + 1) * D + a];
-        if (i > 0 && j + 1 < b.ny) x[a] -= fu[1 * D + a] * rp[(col + b.nx - 1) * D + a];
-        if (j + 1 < b.ny) x[a] -= fu[2 * D + a] * rp[(col + b.nx) * D + a];
-        if (i + 1 < b.nx && j + 1 < b.ny) x[a] -= fu[3 * D + a] * rp[(col + b.nx + 1) * D + a];
-        if (k + 1 < b.nz) x[a] -= fu[4 * D + a] * r1[a];
-        x[a] *= fd[a * D + a];  // 1 / U_aa
-      }
-#pragma unroll
-      for (int a = 0; a < D; ++a) rp[col * D + a] = x[a];
-      if (go >= 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) z[a * N + go] = (V)x[a];
-      }
-    }
-    fetch(L - 1);
-    __syncthreads();
-  }
-}
-
-// Shared-memory staged sweeps (d = 2 boxes whose widest step fits the CTA): every thread copies its
-// own cell's operand block (FwdBlk / BwdBlk) and vector values for the step SG - 1 ahead into a slot
-// of an SG-deep ring with cp.async (one commit group a step) and reads them back after waiting for
-// that step's group, so SG - 1 steps of load latency overlap the step in progress at no register
-// cost, with a few 16-byte copies a cell.  A thread reads only what it copied itself: the wait orders
-// it, and the step keeps one barrier (for the 4-plane ring).  Chunk c of thread t's block in slot s
-// sits at 16-byte element (s * nchunks + c) * blockDim + t (no bank conflicts); the forward result
-// is kept per cell, [cell][d], so the backward sweep stages it with one copy.  The ring is zeroed
-// at launch and padded by `pad` >= (nx + 1) d elements on each side, so every neighbour is read
-// unconditionally: the factor slot of a neighbour outside the box is exactly zero (assembly writes
-// zero there and the factorization never updates it), and the ring holds only finite values.
-template <int B>
-__device__ __forceinline__ void cp_async(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  const size_t g = __cvta_generic_to_global(src);
-  if constexpr (B == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(g) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(g), "n"(B) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-template <class Blk>
-union StagedBlk {
-  Blk b;
-  uint4 u[sizeof(Blk) / 16];
-};
-
-template <class T, class V, int SG, class FT = T>
-__global__ void __launch_bounds__(DENSE_THREADS, 1) ras_fwd_stage_kernel(const long long* __restrict__ cell_off,
-                                                                       const int* __restrict__ dims,
-                                                                       const int* __restrict__ lpt,
-                                                                       const FwdBlk<FT>* __restrict__ blk,
-                                                                       T* __restrict__ loc, int max_cols, int pad,
-                                                                       long long N,
-                                                                       const long long* __restrict__ gmap_p,
-                                                                       const V* __restrict__ r, int stage_off) {
-  constexpr int D = 2, NC = sizeof(FwdBlk<FT>) / 16;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int sd = lpt[blockIdx.x];
-  const SweepBox b = sweep_box(cell_off, dims, sd);
-  const int ring_bytes = ((4 * max_cols * D + 2 * pad) * (int)sizeof(T) + 15) / 16 * 16;
-  T* ring = (T*)smem + pad;  // the padded 4-plane ring: the staged sweeps run only where it fits
-  int* lvl = (int*)(smem + ring_bytes);
-  for (int e = threadIdx.x; e < 4 * b.ncols * D + 2 * pad; e += blockDim.x) ((T*)smem)[e] = T(0);
-  build_tables(b, lvl, nullptr);  // its barriers also order the zeroing
-  const int Tn = blockDim.x, t = threadIdx.x;
-  uint4* sB = (uint4*)(smem + stage_off);                 // [SG][NC][Tn] operand blocks
-  V* sY = (V*)(sB + (size_t)SG * NC * Tn);                // [SG][D][Tn] gathered right-hand side
-  long long* sG = (long long*)(sY + (size_t)SG * D * Tn); // [SG][Tn] cell map entry SG - 1 steps later
-  const FwdBlk<FT>* Bb = blk + b.base;
-  T* Lb = loc + b.base * D;
-  const long long* gm = gmap_p + b.base;
-  auto cnt_of = [&](int L) { return L < b.levels ? lvl[L + 1] - lvl[L] : 0; };
-  // step g into slot g % SG (gg: this thread's cell map entry in step g), and the cell map entry of
-  // step g + SG - 1, which the copies of that step need for the gather
-  auto issue = [&](int g, long long gg) {
-    const int s = g % SG;
-    if (t < cnt_of(g)) {
-      const uint4* src = reinterpret_cast<const uint4*>(Bb + lvl[g] + t);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) cp_async<16>(sB + (s * NC + c) * Tn + t, src + c);
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        if (gg >= 0) cp_async<sizeof(V)>(sY + (s * D + a) * Tn + t, r + a * N + gg);
-        else sY[(s * D + a) * Tn + t] = V(0);
-      }
-    }
-    const int h = g + SG - 1;
-    if (t < cnt_of(h)) cp_async<8>(sG + s * Tn + t, gm + lvl[h] + t);
-    cp_commit();
-  };
-  {  // the first SG - 1 steps' cell map entries, loaded together before any copy is issued
-    long long g0[SG - 1];
-#pragma unroll
-    for (int g = 0; g < SG - 1; ++g) g0[g] = t < cnt_of(g) ? gm[lvl[g] + t] : -1;
-#pragma unroll
-    for (int g = 0; g < SG - 1; ++g) issue(g, g0[g]);
-  }
-  for (int L = 0; L < b.levels; ++L) {
-    cp_wait<SG - 2>();  // step L's group has landed (the SG - 2 later ones may be in flight)
-    const int s = L % SG;
-    issue(L + SG - 1, t < cnt_of(L + SG - 1) ? sG[s * Tn + t] : -1);  // into the slot step L - 1 used
-    if (t < cnt_of(L)) {
-      StagedBlk<FwdBlk<FT>> q;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) q.u[c] = sB[(s * NC + c) * Tn + t];
-      const FT* f = q.b.f;
-      const int i = q.b.ijk & 1023, j = (q.b.ijk >> 10) & 1023, k = q.b.ijk >> 20, col = j * b.nx + i;
-      T* rp = ring + ((k & 3) * b.ncols) * D;
-      const T* r0 = ring + (((k - 1) & 3) * b.ncols + col) * D;
-      T y[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        y[a] = (T)sY[(s * D + a) * Tn + t];
-        y[a] -= fcvt(f[0 * D + a]) * r0[a];
-        y[a] -= fcvt(f[1 * D + a]) * rp[(col - b.nx - 1) * D + a];
-        y[a] -= fcvt(f[2 * D + a]) * rp[(col - b.nx) * D + a];
-        y[a] -= fcvt(f[3 * D + a]) * rp[(col - b.nx + 1) * D + a];
-        y[a] -= fcvt(f[4 * D + a]) * rp[(col - 1) * D + a];
-      }
-      y[1] -= fcvt(f[5 * D]) * y[0];
-      const long long cp = lvl[L] + t;
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        rp[col * D + a] = y[a];
-        Lb[cp * D + a] = y[a];
-      }
-    }
-    __syncthreads();
-  }
-  cp_wait<0>();
-}
-
-// Backward sweep of the staged pair: steps in reverse; each thread's block and its cell's forward
-// result are copied SG - 1 steps ahead.  Nothing a copy needs depends on a staged value, so a step's
-// copies are issued before it waits.
-template <class T, class V, int SG, class FT = T>
-__global__ void __launch_bounds__(DENSE_THREADS, 1) ras_bwd_stage_kernel(const long long* __restrict__ cell_off,
-                                                                       const int* __restrict__ dims,
-                                                                       const int* __restrict__ lpt,
-                                                                       const BwdBlk<FT>* __restrict__ blk,
-                                                                       const T* __restrict__ loc, int max_cols,
-                                                                       int pad, long long N,
-                                                                       V* __restrict__ z, int stage_off) {
-  constexpr int D = 2, NC = sizeof(BwdBlk<FT>) / 16;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int sd = lpt[blockIdx.x];
-  const SweepBox b = sweep_box(cell_off, dims, sd);
-  const int ring_bytes = ((4 * max_cols * D + 2 * pad) * (int)sizeof(T) + 15) / 16 * 16;
-  T* ring = (T*)smem + pad;  // the padded 4-plane ring: the staged sweeps run only where it fits
-  int* lvl = (int*)(smem + ring_bytes);
-  for (int e = threadIdx.x; e < 4 * b.ncols * D + 2 * pad; e += blockDim.x) ((T*)smem)[e] = T(0);
-  build_tables(b, lvl, nullptr);  // its barriers also order the zeroing
-  const int Tn = blockDim.x, t = threadIdx.x;
-  uint4* sB = (uint4*)(smem + stage_off);  // [SG][NC][Tn] operand blocks
-  T* sX = (T*)(sB + (size_t)SG * NC * Tn); // [SG][Tn][D] forward result
-  const BwdBlk<FT>* Bb = blk + b.base;
-  const T* Lb = loc + b.base * D;
-  auto issue = [&](int n) {  // n-th step of the backward order (level levels - 1 - n) into slot n % SG
-    const int L = b.levels - 1 - n, s = n % SG;
-    if (L >= 0 && t < lvl[L + 1] - lvl[L]) {
-      const long long cp = lvl[L] + t;
-      const uint4* src = reinterpret_cast<const uint4*>(Bb + cp);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) cp_async<16>(sB + (s * NC + c) * Tn + t, src + c);
-      cp_async<D * sizeof(T)>(sX + ((size_t)s * Tn + t) * D, Lb + cp * D);
-    }
-    cp_commit();
-  };
-  for (int n = 0; n < SG - 1; ++n) issue(n);
-  for (int n = 0; n < b.levels; ++n) {
-    issue(n + SG - 1);  // into the slot step n - 1 used
-    cp_wait<SG - 1>();  // step n's group has landed
-    const int L = b.levels - 1 - n, s = n % SG;
-    if (t < lvl[L + 1] - lvl[L]) {
-      StagedBlk<BwdBlk<FT>> q;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) q.u[c] = sB[(s * NC + c) * Tn + t];
-      const FT* f = q.b.f;
-      const int i = q.b.ijk & 1023, j = (q.b.ijk >> 10) & 1023, k = q.b.ijk >> 20, col = j * b.nx + i;
-      T* rp = ring + ((k & 3) * b.ncols) * D;
-      const T* r1 = ring + (((k + 1) & 3) * b.ncols + col) * D;
-      T x[D];
-#pragma unroll
-      for (int a = 0; a < D; ++a) x[a] = sX[((size_t)s * Tn + t) * D + a];
-      // U's diagonal block at f[5 d + 0, 1, 2] = 1 / (0,0), (0,1), 1 / (1,1)
-#pragma unroll
-      for (int a = D - 1; a >= 0; --a) {
-        if (a == 0) x[0] -= fcvt(f[5 * D + 1]) * x[1];
-        x[a] -= fcvt(f[0 * D + a]) * rp[(col + 1) * D + a];
-        x[a] -= fcvt(f[1 * D + a]) * rp[(col + b.nx - 1) * D + a];
-        x[a] -= fcvt(f[2 * D + a]) * rp[(col + b.nx) * D + a];
-        x[a] -= fcvt(f[3 * D + a]) * rp[(col + b.nx + 1) * D + a];
-        x[a] -= fcvt(f[4 * D + a]) * r1[a];
-        x[a] *= fcvt(f[a == 0 ? 5 * D : 5 * D + 2]);  // 1 / U_aa
-      }
-#pragma unroll
-      for (int a = 0; a < D; ++a) rp[col * D + a] = x[a];
-      if (q.b.go >= 0) {
-#pragma unroll
-        for (int a = 0; a < D; ++a) z[a * N + q.b.go] = (V)x[a];
-      }
-    }
-    __syncthreads();
-  }
-  cp_wait<0>();
-}
-
 template <class T, int D, class V, class FT = T>
 static fv_status ras_apply_t(const fv_system* s, const V* r, V* z, cudaStream_t st) {
   const Subdomains& S = s->subs;
@@ -1098,67 +652,15 @@ static fv_status ras_apply_t(const fv_system* s, const V* r, V* z, cudaStream_t 
                  FV_K_FP32 * S.fp32;
   {
     ProfScope ps(pf, st);
-    {
-      bool piped = false;
-      if constexpr (D == 2) {
-        const int so = (int)S.stage_off;
-        const FwdBlk<FT>* bf = (const FwdBlk<FT>*)S.blk_f;
-        if (S.stage == 8)
-          ras_fwd_stage_kernel<T, V, 8, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bf, loc, S.max_cols, S.stage_pad, N, S.gmap_p, r, so);
-        else if (S.stage == 6)
-          ras_fwd_stage_kernel<T, V, 6, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bf, loc, S.max_cols, S.stage_pad, N, S.gmap_p, r, so);
-        else if (S.stage == 4)
-          ras_fwd_stage_kernel<T, V, 4, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bf, loc, S.max_cols, S.stage_pad, N, S.gmap_p, r, so);
-        piped = S.stage != 0;
-      }
-      if constexpr (sizeof(T) == 4 || D < 7) {
-        if (S.dense_single && !piped) {
-          ras_fwd_pipe_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
-              S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p,
-              S.ijk, r);
-          piped = true;
-        }
-      }
-      if (!piped)
-        ras_fwd_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
-            S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p, r);
-    }
+    ras_fwd_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
+        S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p, r);
   }
   FV_CUDA(cudaGetLastError());
   {
     ProfScope ps(pb, st);
-    {
-      bool piped = false;
-      if constexpr (D == 2) {
-        const int so = (int)S.stage_off;
-        const BwdBlk<FT>* bb = (const BwdBlk<FT>*)S.blk_b;
-        if (S.stage == 8)
-          ras_bwd_stage_kernel<T, V, 8, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bb, loc, S.max_cols, S.stage_pad, N, z, so);
-        else if (S.stage == 6)
-          ras_bwd_stage_kernel<T, V, 6, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bb, loc, S.max_cols, S.stage_pad, N, z, so);
-        else if (S.stage == 4)
-          ras_bwd_stage_kernel<T, V, 4, FT><<<S.count, S.dense_threads, S.stage_smem, st>>>(
-              S.cell_off, S.dims, S.lpt, bb, loc, S.max_cols, S.stage_pad, N, z, so);
-        piped = S.stage != 0;
-      }
-      if constexpr (sizeof(T) == 4 || D < 7) {
-        if (S.dense_single && !piped) {
-          ras_bwd_pipe_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
-              S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p,
-              S.owned_p, S.ijk, z);
-          piped = true;
-        }
-      }
-      if (!piped)
-        ras_bwd_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
-            S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p,
-            S.owned_p, z);
-    }
+    ras_bwd_kernel<T, D, V, FT><<<S.count, S.dense_threads, S.smem, st>>>(
+        S.cell_off, S.dims, S.lpt, (const FT*)S.F, loc, (T*)S.ring, S.ring_in_smem, S.max_cols, N, S.gmap_p, S.owned_p,
+        z);
   }
   FV_CUDA(cudaGetLastError());
   return FV_OK;
@@ -1170,18 +672,6 @@ template <class T, int D, class FT = T>
 static fv_status set_smem_attr(int limit) {
   FV_CUDA(cudaFuncSetAttribute(ras_fwd_kernel<T, D, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   FV_CUDA(cudaFuncSetAttribute(ras_bwd_kernel<T, D, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  if constexpr (sizeof(T) == 4 || D < 7) {
-    FV_CUDA(cudaFuncSetAttribute(ras_fwd_pipe_kernel<T, D, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_bwd_pipe_kernel<T, D, T, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  }
-  if constexpr (D == 2) {
-    FV_CUDA(cudaFuncSetAttribute(ras_fwd_stage_kernel<T, T, 8, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_bwd_stage_kernel<T, T, 8, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_fwd_stage_kernel<T, T, 6, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_bwd_stage_kernel<T, T, 6, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_fwd_stage_kernel<T, T, 4, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-    FV_CUDA(cudaFuncSetAttribute(ras_bwd_stage_kernel<T, T, 4, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  }
   return FV_OK;
 }
 
@@ -1190,16 +680,26 @@ fv_status sweeps_smem_attr(const fv_system* s) {
   int dev = 0, limit = 0;
   FV_CUDA(cudaGetDevice(&dev));
   FV_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (S.smem > (size_t)limit || S.stage_smem > (size_t)limit)
+  if (S.st.on) return FV_OK;
+  if (S.smem > (size_t)limit)
     return set_error("fv_assemble_system: sweep tables exceed shared memory"), FV_EINVAL;
   if (S.bf16) return S.d == 2 ? set_smem_attr<float, 2, __nv_bfloat16>(limit) : set_smem_attr<float, 7, __nv_bfloat16>(limit);
   if (S.d == 2) return S.fp32 ? set_smem_attr<float, 2>(limit) : set_smem_attr<double, 2>(limit);
   return S.fp32 ? set_smem_attr<float, 7>(limit) : set_smem_attr<double, 7>(limit);
 }
 
+// kernel timing of the streamed sweeps (one launch for both directions): the forward category
+static int sweep_category(const fv_system* s) {
+  return (s->kind == FV_VTBE ? FV_K_RAS_FWD_VTBE : FV_K_RAS_FWD_PPBE) + FV_K_COARSE * s->level + FV_K_FP32 * s->subs.fp32;
+}
+
 fv_status ras_apply(const fv_system* s, const double* r, double* z, cudaStream_t st) {
   const Subdomains& S = s->subs;
   if (S.fp32) return set_error("ras_apply: FP32 factors need FP32 vectors"), FV_EINVAL;
+  if (S.st.on) {
+    ProfScope ps(sweep_category(s), st);
+    return ras_stream64(s, 1, r, 0, z, 0, S.st.loc, st);
+  }
   if (S.d == 2) return ras_apply_t<double, 2, double>(s, r, z, st);
   return ras_apply_t<double, 7, double>(s, r, z, st);
 }
@@ -1207,6 +707,10 @@ fv_status ras_apply(const fv_system* s, const double* r, double* z, cudaStream_t
 static fv_status ras_apply32(const fv_system* s, const float* r, float* z, cudaStream_t st) {
   const Subdomains& S = s->subs;
   if (!S.fp32) return set_error("ras_apply32: FP64 factors need FP64 vectors"), FV_EINVAL;
+  if (S.st.on) {
+    ProfScope ps(sweep_category(s), st);
+    return ras_stream32(s, r, z, st);
+  }
   if (S.bf16)
     return S.d == 2 ? ras_apply_t<float, 2, float, __nv_bfloat16>(s, r, z, st)
                     : ras_apply_t<float, 7, float, __nv_bfloat16>(s, r, z, st);
