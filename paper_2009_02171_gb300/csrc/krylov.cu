@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -50,6 +51,9 @@ struct KrylovT {
   double* hhost = nullptr;  // pinned [3][KMAX]
   ArnoldiDev* ad = nullptr; // device-driven solves
   unsigned* ticket = nullptr; // last-block counter of the fused reductions (returns to 0 after each use)
+  unsigned* bar = nullptr;    // [2] grid barrier of the one-launch Gram-Schmidt step: arrivals, generation
+  int *err = nullptr, *err_dev = nullptr;  // mapped host word: a grid barrier ran out
+  int sms = 0, smem = 0;
 };
 
 struct Krylov {
@@ -59,8 +63,8 @@ struct Krylov {
 
 template <class T>
 static void free_kt(KrylovT<T>& k) {
-  cudaFree(k.V), cudaFree(k.Z), cudaFree(k.w), cudaFree(k.r), cudaFree(k.part), cudaFree(k.h), cudaFree(k.ad), cudaFree(k.ticket);
-  cudaFreeHost(k.hhost);
+  cudaFree(k.V), cudaFree(k.Z), cudaFree(k.w), cudaFree(k.r), cudaFree(k.part), cudaFree(k.h), cudaFree(k.ad), cudaFree(k.ticket), cudaFree(k.bar);
+  cudaFreeHost(k.hhost), cudaFreeHost(k.err);
   k = KrylovT<T>();
 }
 
@@ -79,6 +83,9 @@ template <>
 KrylovT<float>& kt<float>(Krylov* k) { return k->f; }
 
 template <class T>
+static fv_status gs_limits(KrylovT<T>& k);
+
+template <class T>
 static fv_status ensure_krylov(const fv_system* s, int m) {
   fv_system* sm = const_cast<fv_system*>(s);
   if (!sm->kry) sm->kry = new Krylov();
@@ -93,11 +100,15 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
       cudaMalloc(&k.h, 3 * KMAX * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&k.ad, sizeof(ArnoldiDev)) != cudaSuccess || cudaMalloc(&k.ticket, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(k.ticket, 0, sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&k.bar, 2 * sizeof(unsigned)) != cudaSuccess || cudaMemset(k.bar, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
+      cudaHostAlloc((void**)&k.err, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer((void**)&k.err_dev, k.err, 0) != cudaSuccess ||
       cudaMallocHost(&k.hhost, 3 * KMAX * sizeof(double)) != cudaSuccess) {
     free_kt(k);
     return set_error("fv_gmres_solve: device allocation of the Krylov basis failed"), FV_ENOMEM;
   }
-  return FV_OK;
+  *k.err = 0;
+  return gs_limits<T>(k);
 }
 
 // ------------------------------------------------------------------ vector kernels
@@ -146,21 +157,29 @@ __device__ __forceinline__ void block_store_n(double (&acc)[NA], int nv, double*
   }
 }
 
+// the rotation (c, s) that takes (a, b) to (den, 0); returns den
+__device__ __forceinline__ double givens_rotation(double a, double b, double& c, double& s) {
+  const double big = fmax(fabs(a), fabs(b));
+  const double den = big > 1e-140 && big < 1e140 ? sqrt(a * a + b * b) : hypot(a, b);
+  const double rden = den > 0.0 ? 1.0 / den : 0.0;
+  c = den > 0.0 ? a * rden : 1.0, s = b * rden;
+  return den;
+}
+
 // Givens update of column j of the device-driven Arnoldi (thread 0 of one block):
-// h = h1 + h2 (CGS2), h_{j+1,j} = sqrt(nrm2); previous rotations, new rotation,
-// right-hand side update; scale = 1 / h_{j+1,j}
-__device__ void givens_update(int j, const double* __restrict__ h, double nrm2, ArnoldiDev* ad) {
+// h = h1 + h2 (CGS2), h_{j+1,j} = hn; previous rotations, new rotation,
+// right-hand side update; scale = rhn = 1 / hn (0 for hn = 0)
+__device__ void givens_update(int j, const double* h, double hn, double rhn, ArnoldiDev* ad) {
   double col[KMAX + 1];
   for (int i = 0; i <= j; ++i) col[i] = h[i] + h[KMAX + i];
-  const double hn = sqrt(nrm2);
   col[j + 1] = hn;
   for (int i = 0; i < j; ++i) {
     const double a = ad->cs[i] * col[i] + ad->sn[i] * col[i + 1];
     col[i + 1] = -ad->sn[i] * col[i] + ad->cs[i] * col[i + 1];
     col[i] = a;
   }
-  const double den = hypot(col[j], col[j + 1]);
-  const double c = den > 0.0 ? col[j] / den : 1.0, s = den > 0.0 ? col[j + 1] / den : 0.0;
+  double c, s;
+  const double den = givens_rotation(col[j], col[j + 1], c, s);
   ad->cs[j] = c, ad->sn[j] = s;
   col[j] = den;
   ad->g[j + 1] = -s * ad->g[j];
@@ -168,7 +187,18 @@ __device__ void givens_update(int j, const double* __restrict__ h, double nrm2, 
   for (int i = 0; i <= j; ++i) ad->H[j * KMAX + i] = col[i];
   if (!(den > 0.0) && ad->k_eff > j) ad->k_eff = j;              // no usable column j
   else if (!(hn > 0.0) && ad->k_eff > j + 1) ad->k_eff = j + 1;  // lucky breakdown after column j
-  ad->scale = hn > 0.0 ? 1.0 / hn : 0.0;
+  ad->scale = rhn;
+}
+
+// y = H^{-1} g on the first min(m, k_eff) columns (back substitution), zero beyond
+__device__ void least_squares(int m, ArnoldiDev* ad) {
+  const int kk = m < ad->k_eff ? m : ad->k_eff;
+  for (int i = KMAX - 1; i >= kk; --i) ad->y[i] = 0.0;
+  for (int i = kk - 1; i >= 0; --i) {
+    double s = ad->g[i];
+    for (int q = i + 1; q < kk; ++q) s -= ad->H[q * KMAX + i] * ad->y[q];
+    ad->y[i] = s / ad->H[i * KMAX + i];
+  }
 }
 
 // sum of the nb partials p[0..nb) by one warp in a fixed order; the loads of a lane are issued
@@ -347,7 +377,10 @@ __global__ void __launch_bounds__(RTHREADS, (NV > (sizeof(T) == 8 ? 18 : 14) ? 1
   for (int v = wid; v < nvv; v += nw) out[v] = last_block_sum(part + v * gridDim.x, (int)gridDim.x, lane);
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (mode == 2 && ad) givens_update(gj, hg, out[0], ad);
+    if (mode == 2 && ad) {
+      const double hn = sqrt(out[0]);
+      givens_update(gj, hg, hn, hn > 0.0 ? 1.0 / hn : 0.0, ad);
+    }
     *ticket = 0u;
   }
 }
@@ -364,6 +397,321 @@ static int cgs_blocks(long long n, bool vec) {
 template <class T>
 static bool cgs_vec(long long n, const T* V, const T* w) {
   return n % Vec16<T>::L == 0 && (reinterpret_cast<uintptr_t>(V) & 15) == 0 && (reinterpret_cast<uintptr_t>(w) & 15) == 0;
+}
+
+// ------------------------------------------------------------------ Gram-Schmidt step in one launch
+// One Arnoldi step's orthogonalization (one or two classical Gram-Schmidt passes), norm, Givens update and the
+// next basis vector, v = w / ||w||, with a grid barrier between its reductions, for vectors whose slice per SM
+// fits in shared memory: w is read from memory once and kept there, only the basis is read again.  At the sizes
+// of the coarse level (n = 393,216 FP32: 1.5 MB a vector, all in L2) the separate passes were bound by their
+// launches, drains and the FP64 arithmetic of the block reductions (five dependent DADDs a warp and value, 16
+// cycles of the SM's FP64 pipe each); here a value's 512 partial sums go through shared memory, where one warp
+// adds 16 a lane before its butterfly, a quarter of the operations.  Measured: see gs_step().
+constexpr int GS_THREADS = 512;          // threads a block at most
+// FP64: 512, half of them above 16 basis vectors (registers).  FP32: 256, since every thread's partial sums are
+// converted to FP64 on the slow pipe (coarse level, 5 vectors: 24.6 us with 512 threads, see gs_step())
+__host__ __device__ constexpr int gs_threads(int nv, int es) { return es == 4 || nv > 16 ? GS_THREADS / 2 : GS_THREADS; }
+constexpr int GS_CHUNK = 8;              // values reduced together: [GS_CHUNK][GS_THREADS] doubles of shared memory
+constexpr unsigned GS_SPINS = 1u << 24;  // bound of a barrier's wait
+
+struct GsArgs {
+  long long n, slice;   // elements; elements a block
+  int keep;             // the block's slice of the basis is kept in shared memory for the later passes
+  int passes;           // Gram-Schmidt passes (0: norm and scaling alone)
+  int start;            // 1: the norm starts a cycle (ad->g = ||w|| e_1)
+  int last;             // 1: after this column solve the least-squares problem into ad->y
+  int gj;
+  double* part;         // [3][KMAX][blocks]
+  double* h;            // [3][KMAX]: the two passes' coefficients, ||w||^2
+  ArnoldiDev* ad;       // device-driven solves
+  unsigned* bar;
+  int* err;
+};
+
+// all blocks (co-resident: cooperative launch) meet; bounded, a wait that runs out is reported through err
+__device__ __forceinline__ void grid_barrier(unsigned* bar, int* err) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned gen, cur;
+    asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(gen) : "l"(bar + 1) : "memory");
+    __threadfence();
+    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+      bar[0] = 0;
+      __threadfence();
+      atomicAdd(bar + 1, 1u);
+    } else {
+      unsigned t = 0;
+      do {
+        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(bar + 1) : "memory");
+      } while (cur == gen && ++t < GS_SPINS);
+      if (cur == gen) *err = 1;
+    }
+    __threadfence();
+  }
+  __syncthreads();
+}
+
+// sums of acc[0..nv) over the block into part[v * gridDim.x + blockIdx.x], fixed order
+template <int NA, int TH>
+__device__ __forceinline__ void gs_reduce(double (&acc)[NA], int nv, double* red, double* part) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int v0 = 0; v0 < NA; v0 += GS_CHUNK) {
+    if (v0 >= nv) break;
+    if (v0) __syncthreads();
+#pragma unroll
+    for (int u = 0; u < GS_CHUNK; ++u)
+      if (v0 + u < NA && v0 + u < nv) red[u * TH + threadIdx.x] = acc[v0 + u < NA ? v0 + u : 0];
+    __syncthreads();
+    if (wid < GS_CHUNK && v0 + wid < nv) {
+      const double* q = red + wid * TH + lane;
+      double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+      for (int u = 0; u < TH / 32; u += 2) t0 += q[32 * u], t1 += q[32 * (u + 1)];
+      const double t = warp_sum(t0 + t1);
+      if (lane == 0) part[(v0 + wid) * gridDim.x + blockIdx.x] = t;
+    }
+  }
+}
+
+// the grid's sums out[0..nv) from the blocks' partials, the same order in every block
+template <int TH>
+__device__ __forceinline__ void gs_total(const double* part, int nv, double* out) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int v = wid; v < nv; v += TH / 32) {
+    const double t = last_block_sum(part + v * gridDim.x, (int)gridDim.x, lane);
+    if (lane == 0) out[v] = t;
+  }
+  __syncthreads();
+}
+
+template <int NV, class T>
+__global__ void __launch_bounds__(gs_threads(NV, sizeof(T)), 1) gs_kernel(GsArgs A, const T* __restrict__ V, const T* w, T* vout) {
+  constexpr int NA = NV > 0 ? NV : 1, L = Vec16<T>::L, TH = gs_threads(NV, sizeof(T));
+  constexpr bool F32 = sizeof(T) == 4;
+  extern __shared__ __align__(16) unsigned char gs_smem[];
+  double* red = reinterpret_cast<double*>(gs_smem);
+  T* ws = reinterpret_cast<T*>(gs_smem + GS_CHUNK * GS_THREADS * sizeof(double));
+  T* vs = ws + A.slice;  // [NV][slice] when A.keep
+  __shared__ double tot[NA], coef[NA];
+  __shared__ T hs[NA];
+  // what the Givens update of block 0 needs of the earlier columns, fetched now
+  __shared__ double rot[2][NA], Hs[NA * NA], gj0;
+  const bool givens = blockIdx.x == 0 && A.ad && !A.start;
+  if (givens) {
+    if (threadIdx.x < A.gj) rot[0][threadIdx.x] = A.ad->cs[threadIdx.x], rot[1][threadIdx.x] = A.ad->sn[threadIdx.x];
+    if (threadIdx.x == TH - 1) gj0 = A.ad->g[A.gj];
+    if (A.last)
+      for (int e = threadIdx.x; e < A.gj * A.gj; e += TH) Hs[e / A.gj * NA + e % A.gj] = A.ad->H[e / A.gj * KMAX + e % A.gj];
+  }
+  const long long n = A.n, b0 = blockIdx.x * A.slice;
+  const int len = (int)(n - b0 < A.slice ? (n > b0 ? n - b0 : 0) : A.slice);
+  const bool vec = n % L == 0 && ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
+  const int ng = vec ? len / L : 0;
+  const T* Vb = V + b0;
+  const T* wb = w + b0;
+  double acc[NA];
+  T cur[NA];
+  // FP32 products are summed in FP32 for at most 32 elements of a thread, then in FP64
+  auto clear = [&]() {
+#pragma unroll
+    for (int v = 0; v < NA; ++v) acc[v] = 0.0, cur[v] = T(0);
+  };
+  auto flush = [&]() {
+    if constexpr (F32)
+#pragma unroll
+      for (int v = 0; v < NA; ++v) acc[v] += (double)cur[v], cur[v] = T(0);
+  };
+  auto add = [&](int v, T a, T b) {
+    if constexpr (F32) cur[v] += a * b;
+    else acc[v] += a * b;
+  };
+  // one pass over the slice.  sub: w -= V h;  dots: V^T w, else w^T w;  first: w comes from memory
+  auto pass = [&](auto first, bool sub, bool dots) {
+    clear();
+    int cnt = 0;
+#pragma unroll(NV <= 8 ? 2 : 1)
+    for (int g = threadIdx.x; g < ng; g += TH) {
+      const int e = g * L;
+      T we[L];
+      if constexpr (decltype(first)::value) Vec16<T>::load(wb + e, we);
+      else Vec16<T>::load(ws + e, we);
+      T vv[NA][L];
+      if (decltype(first)::value || !A.keep) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Vec16<T>::ldg(Vb + v * n + e, vv[v]);
+        if (A.keep) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Vec16<T>::store(vs + v * (int)A.slice + e, vv[v]);
+        }
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Vec16<T>::load(vs + v * (int)A.slice + e, vv[v]);
+      }
+      if (sub) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int l = 0; l < L; ++l) we[l] -= hs[v] * vv[v][l];
+      }
+      if (decltype(first)::value || sub) Vec16<T>::store(ws + e, we);
+      if (dots) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int l = 0; l < L; ++l) add(v, vv[v][l], we[l]);
+      } else {
+#pragma unroll
+        for (int l = 0; l < L; ++l) add(0, we[l], we[l]);
+      }
+      cnt += L;
+      if (F32 && cnt >= 32) flush(), cnt = 0;
+    }
+    for (int e = ng * L + threadIdx.x; e < len; e += TH) {  // unaligned vectors, or a ragged end
+      T we;
+      if constexpr (decltype(first)::value) we = wb[e];
+      else we = ws[e];
+      if (sub) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) we -= hs[v] * Vb[v * n + e];
+      }
+      if (decltype(first)::value || sub) ws[e] = we;
+      if (dots) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) add(v, Vb[v * n + e], we);
+      } else {
+        add(0, we, we);
+      }
+      if (F32 && ++cnt >= 32) flush(), cnt = 0;
+    }
+    flush();
+  };
+  double* part = A.part;
+  if (A.passes > 0) {
+    pass(std::true_type(), false, true);
+    gs_reduce<NA, TH>(acc, NV, red, part);
+    for (int q = 0; q < A.passes; ++q) {
+      grid_barrier(A.bar, A.err);
+      gs_total<TH>(part, NV, tot);
+      if (threadIdx.x < NV) {
+        hs[threadIdx.x] = (T)tot[threadIdx.x];
+        coef[threadIdx.x] = (q ? coef[threadIdx.x] : 0.0) + tot[threadIdx.x];
+        if (blockIdx.x == 0) A.h[q * KMAX + threadIdx.x] = tot[threadIdx.x];
+      }
+      __syncthreads();
+      part += KMAX * gridDim.x;
+      const bool more = q + 1 < A.passes;
+      pass(std::false_type(), true, more);
+      gs_reduce<NA, TH>(acc, more ? NV : 1, red, part);
+    }
+    if (A.passes == 1 && blockIdx.x == 0 && threadIdx.x < NV) A.h[KMAX + threadIdx.x] = 0.0;
+  } else {
+    pass(std::true_type(), false, false);
+    gs_reduce<NA, TH>(acc, 1, red, part);
+  }
+  grid_barrier(A.bar, A.err);
+  gs_total<TH>(part, 1, tot);
+  // one thread takes the square root and the reciprocal: on the FP64 pipe (16 cycles a warp instruction) every
+  // warp doing so cost more than a pass over the basis
+  __shared__ T inv;
+  double hn = 0.0, rhn = 0.0;
+  if (threadIdx.x == 0) {
+    hn = sqrt(tot[0]);
+    rhn = hn > 0.0 ? 1.0 / hn : 0.0;
+    inv = (T)rhn;
+  }
+  if (vout) {
+    __syncthreads();
+    const T a = inv;
+    T* vb = vout + b0;
+    for (int g = threadIdx.x; g < ng; g += TH) {
+      T we[L];
+      Vec16<T>::load(ws + g * L, we);
+  #pragma unroll
+      for (int l = 0; l < L; ++l) we[l] *= a;
+      Vec16<T>::store(vb + g * L, we);
+    }
+    for (int e = ng * L + threadIdx.x; e < len; e += TH) vb[e] = a * ws[e];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    A.h[2 * KMAX] = tot[0];
+    if (A.ad && A.start) {
+      for (int i = 0; i <= KMAX; ++i) A.ad->g[i] = 0.0;
+      A.ad->g[0] = hn;
+      A.ad->scale = rhn;
+      A.ad->k_eff = hn > 0.0 ? KMAX : 0;
+    } else if (A.ad) {
+      // as givens_update(), from shared memory
+      const int j = A.gj;
+      double c0 = coef[0];
+      for (int i = 0; i < j; ++i) {
+        const double c1 = coef[i + 1 < NA ? i + 1 : 0];
+        coef[i] = rot[0][i] * c0 + rot[1][i] * c1;
+        c0 = -rot[1][i] * c0 + rot[0][i] * c1;
+      }
+      double c, s;
+      const double den = givens_rotation(c0, hn, c, s);
+      coef[j] = den;
+      for (int i = 0; i <= j; ++i) A.ad->H[j * KMAX + i] = coef[i];
+      A.ad->cs[j] = c, A.ad->sn[j] = s;
+      A.ad->g[j + 1] = -s * gj0;
+      A.ad->g[j] = c * gj0;
+      int k_eff = A.ad->k_eff;
+      if (!(den > 0.0) && k_eff > j) k_eff = j;              // no usable column j
+      else if (!(hn > 0.0) && k_eff > j + 1) k_eff = j + 1;  // lucky breakdown after column j
+      A.ad->k_eff = k_eff;
+      A.ad->scale = rhn;
+      if (A.last) {
+        const int kk = min(j + 1, k_eff);
+        double y[NA];
+        for (int i = KMAX - 1; i >= kk; --i) A.ad->y[i] = 0.0;
+#pragma unroll
+        for (int i = NA - 1; i >= 0; --i) {
+          if (i >= kk) continue;
+          double t = i == j ? c * gj0 : A.ad->g[i];
+#pragma unroll
+          for (int q = i + 1; q < NA; ++q)
+            if (q < kk) t -= (q == j ? coef[i] : Hs[q * NA + i]) * y[q];
+          y[i] = t / (i == j ? coef[i] : Hs[i * NA + i]);
+          A.ad->y[i] = y[i];
+        }
+      }
+    }
+  }
+}
+
+template <int NV, class T>
+static const void* gs_kernel_ptr() { return reinterpret_cast<const void*>(&gs_kernel<NV, T>); }
+
+template <class T, int... I>
+static const void* gs_kernel_of(int nv, std::integer_sequence<int, I...>) {
+  using F = const void* (*)();
+  static const F table[] = {&gs_kernel_ptr<I, T>...};
+  return table[nv]();
+}
+
+template <class T>
+static fv_status gs_limits(KrylovT<T>& k) {
+  int dev = 0, limit = 0;
+  FV_CUDA(cudaGetDevice(&dev));
+  FV_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  FV_CUDA(cudaDeviceGetAttribute(&k.sms, cudaDevAttrMultiProcessorCount, dev));
+  k.smem = limit - 12 * 1024;  // less the kernel's static shared memory
+  for (int v = 0; v < KMAX; ++v)
+    FV_CUDA(cudaFuncSetAttribute(gs_kernel_of<T>(v, std::make_integer_sequence<int, KMAX>{}),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem));
+  return FV_OK;
+}
+
+// Blocks and shared memory of the one-launch step for vectors of n; 0 blocks: the slice does not fit (the separate
+// passes below stream such vectors at HBM rate: FP64 above 3.7M, FP32 above 7.4M elements).  At least 1024 elements
+// a block: fewer only add partials and arrivals at the barrier.
+template <class T>
+static int gs_blocks(const KrylovT<T>& k, long long n, long long* slice, size_t* smem) {
+  const long long blocks = std::max<long long>(1, std::min<long long>(k.sms, n / 1024));
+  *slice = ((n + blocks - 1) / blocks + 15) / 16 * 16;
+  *smem = GS_CHUNK * GS_THREADS * sizeof(double) + (size_t)*slice * sizeof(T);
+  return *smem <= (size_t)k.smem ? (int)((n + *slice - 1) / *slice) : 0;
 }
 
 struct CgsFuse {
@@ -407,6 +755,97 @@ __global__ void reduce_kernel(const double* __restrict__ part, int nb, int nv, d
   }
 }
 
+// beta = ||r|| from the norm partials; g = (beta, 0, ...); scale = 1/beta
+__global__ void start_kernel(const double* __restrict__ part, int nb, ArnoldiDev* ad) {
+  const int lane = threadIdx.x;
+  double t = 0.0;
+  for (int b = lane; b < nb; b += 32) t += part[b];
+  t = warp_sum(t);
+  if (lane == 0) {
+    const double beta = sqrt(t);
+    for (int i = 0; i <= KMAX; ++i) ad->g[i] = 0.0;
+    ad->g[0] = beta;
+    ad->scale = beta > 0.0 ? 1.0 / beta : 0.0;
+    ad->k_eff = beta > 0.0 ? KMAX : 0;
+  }
+}
+
+__global__ void lsq_kernel(int m, ArnoldiDev* ad) {
+  if (threadIdx.x == 0) least_squares(m, ad);
+}
+
+template <class T>
+__global__ void dscale_kernel(long long n, const T* __restrict__ x, const double* __restrict__ scale, T* __restrict__ out) {
+  const T a = (T)*scale;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
+    out[e] = a * x[e];
+}
+
+// out = x / sqrt(*nrm2) (zero for a zero norm)
+template <class T>
+__global__ void rscale_kernel(long long n, const T* __restrict__ x, const double* __restrict__ nrm2, T* __restrict__ out) {
+  const double hn = sqrt(*nrm2);
+  const T a = (T)(hn > 0.0 ? 1.0 / hn : 0.0);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
+    out[e] = a * x[e];
+}
+
+static int vblocks(long long n) { return (int)std::min<long long>(std::max<long long>((n + 255) / 256, 1), 152LL * 16); }
+
+// One Arnoldi step's orthogonalization of k.w against the first nv basis vectors (`passes` passes) and the next basis
+// vector into vout (null: none); with ad, the Givens update of column nv - 1 (last: and the least-squares solve).
+// nv = 0: the norm of w and w / ||w|| (with ad: the start of a cycle).  One cooperative launch where the slices of w
+// fit in shared memory, else the separate passes.
+// A step against the separate passes, us on GB300 (mean over a cycle): FP32 coarse level 6x32^3 (one pass) 28.5 -> 21,
+// 6x64^2x48 59 -> 38; FP32 6x64^3 72 -> 55; FP64 (two passes) 6x45^2x39 218 -> 137, 6x16^3 64 -> 40.
+template <class T>
+static fv_status gs_step(const KrylovT<T>& k, int nv, long long n, const T* w, T* vout, int passes, ArnoldiDev* ad,
+                         bool last, cudaStream_t st) {
+  GsArgs a{};
+  size_t smem = 0;
+  const int blocks = gs_blocks<T>(k, n, &a.slice, &smem);
+  if (blocks) {
+    // basis and w in shared memory: short vectors (the coarse level) read nothing twice
+    const size_t keep = (size_t)nv * a.slice * sizeof(T);
+    a.keep = nv > 0 && n % Vec16<T>::L == 0 && smem + keep <= (size_t)k.smem;
+    if (a.keep) smem += keep;
+    a.n = n, a.passes = nv > 0 ? passes : 0, a.start = nv == 0, a.last = last, a.gj = nv - 1;
+    a.part = k.part, a.h = k.h, a.ad = ad, a.bar = k.bar, a.err = k.err_dev;
+    const T* V = nv > 0 ? k.V : w;
+    void* args[] = {&a, &V, &w, &vout};
+    FV_CUDA(cudaLaunchCooperativeKernel(gs_kernel_of<T>(nv, std::make_integer_sequence<int, KMAX>{}), dim3(blocks),
+                                        dim3(gs_threads(nv, sizeof(T))), args, smem, st));
+    return FV_OK;
+  }
+  T* wm = const_cast<T*>(w);
+  if (nv == 0) {
+    cgs_launch<T>(0, n, w, nullptr, wm, k.part, 2, st);
+    const int nb = cgs_blocks<T>(n, cgs_vec<T>(n, w, w));
+    if (ad) start_kernel<<<1, 32, 0, st>>>(k.part, nb, ad);
+    else reduce_kernel<<<1, RTHREADS, 0, st>>>(k.part, nb, 1, k.h + 2 * KMAX);
+  } else {
+    CgsFuse f;
+    f.ticket = k.ticket;
+    f.out = k.h;
+    cgs_launch<T>(nv, n, k.V, nullptr, wm, k.part, 0, st, f);
+    if (passes == 2) {
+      f.out = k.h + KMAX;
+      cgs_launch<T>(nv, n, k.V, k.h, wm, k.part, 1, st, f);
+    } else if (nv == 1) {
+      FV_CUDA(cudaMemsetAsync(k.h + KMAX, 0, KMAX * sizeof(double), st));
+    }
+    f.out = k.h + 2 * KMAX, f.ad = ad, f.gj = nv - 1, f.hg = k.h;
+    cgs_launch<T>(nv, n, k.V, passes == 2 ? k.h + KMAX : k.h, wm, k.part, 2, st, f);
+    if (last && ad) lsq_kernel<<<1, 32, 0, st>>>(nv, ad);
+  }
+  if (vout) {
+    if (ad) dscale_kernel<T><<<vblocks(n), 256, 0, st>>>(n, w, &ad->scale, vout);
+    else rscale_kernel<T><<<vblocks(n), 256, 0, st>>>(n, w, k.h + 2 * KMAX, vout);
+  }
+  FV_CUDA(cudaGetLastError());
+  return FV_OK;
+}
+
 template <class T, class U>
 __global__ void axpby_kernel(long long n, double a, const U* __restrict__ x, double b, const T* y, T* out) {
   const T at = (T)a, bt = (T)b;
@@ -444,8 +883,6 @@ static void update_dispatch(int nv, int blocks, long long n, const T* Z, const C
   table[nv](blocks, n, Z, y, x, st);
 }
 
-static int vblocks(long long n) { return (int)std::min<long long>(std::max<long long>((n + 255) / 256, 1), 152LL * 16); }
-
 fv_status axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st) {
   ProfScope ps(FV_K_VEC, st);
   axpby_kernel<double, double><<<vblocks(n), 256, 0, st>>>(n, a, x, b, y, out);
@@ -482,11 +919,10 @@ static fv_status axpby_t(long long n, double a, const T* x, double b, const T* y
   return FV_OK;
 }
 
+// ||x||, and x / ||x|| into vout (null: none)
 template <class T>
-static fv_status norm2(KrylovT<T>& k, long long n, const T* x, cudaStream_t st, double* out) {
-  cgs_launch<T>(0, n, x, nullptr, const_cast<T*>(x), k.part, 2, st);
-  reduce_kernel<<<1, RTHREADS, 0, st>>>(k.part, cgs_blocks<T>(n, cgs_vec<T>(n, x, x)), 1, k.h + 2 * KMAX);
-  FV_CUDA(cudaGetLastError());
+static fv_status norm2(KrylovT<T>& k, long long n, const T* x, T* vout, cudaStream_t st, double* out) {
+  if (fv_status rc = gs_step<T>(k, 0, n, x, vout, 0, nullptr, false, st)) return rc;
   FV_CUDA(cudaMemcpyAsync(k.hhost, k.h + 2 * KMAX, sizeof(double), cudaMemcpyDeviceToHost, st));
   FV_CUDA(cudaStreamSynchronize(st));
   *out = std::sqrt(k.hhost[0]);
@@ -516,40 +952,6 @@ fv_status precond_t<float>(const fv_system* s, const float* r, float* z, cudaStr
 }
 
 // ------------------------------------------------------------------ device-driven FGMRES
-// beta = ||r|| from the norm partials; g = (beta, 0, ...); scale = 1/beta
-__global__ void start_kernel(const double* __restrict__ part, int nb, ArnoldiDev* ad) {
-  const int lane = threadIdx.x;
-  double t = 0.0;
-  for (int b = lane; b < nb; b += 32) t += part[b];
-  t = warp_sum(t);
-  if (lane == 0) {
-    const double beta = sqrt(t);
-    for (int i = 0; i <= KMAX; ++i) ad->g[i] = 0.0;
-    ad->g[0] = beta;
-    ad->scale = beta > 0.0 ? 1.0 / beta : 0.0;
-    ad->k_eff = beta > 0.0 ? KMAX : 0;
-  }
-}
-
-// y = H^{-1} g on the first min(m, k_eff) columns (back substitution), zero beyond
-__global__ void lsq_kernel(int m, ArnoldiDev* ad) {
-  if (threadIdx.x != 0) return;
-  const int kk = m < ad->k_eff ? m : ad->k_eff;
-  for (int i = KMAX - 1; i >= 0; --i) ad->y[i] = 0.0;
-  for (int i = kk - 1; i >= 0; --i) {
-    double s = ad->g[i];
-    for (int q = i + 1; q < kk; ++q) s -= ad->H[q * KMAX + i] * ad->y[q];
-    ad->y[i] = s / ad->H[i * KMAX + i];
-  }
-}
-
-template <class T>
-__global__ void dscale_kernel(long long n, const T* __restrict__ x, const double* __restrict__ scale, T* __restrict__ out) {
-  const T a = (T)*scale;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-    out[e] = a * x[e];
-}
-
 // x = sum_v y_v Z_v with y in device memory
 template <int NV, class T>
 __global__ void dupdate_kernel(long long n, const T* __restrict__ Z, const double* __restrict__ y, T* __restrict__ x) {
@@ -591,35 +993,18 @@ static fv_status gmres_fixed_t(const fv_system* s, const T* b, T* x, int m, cuda
   const bool once = s->pc.inner_gs_passes == 1;
   {
     ProfScope ps(FV_K_CGS + lvl, st);
-    if (once) FV_CUDA(cudaMemsetAsync(k.h + KMAX, 0, KMAX * sizeof(double), st));
-    cgs_launch<T>(0, n, b, nullptr, const_cast<T*>(b), k.part, 2, st);
-    start_kernel<<<1, 32, 0, st>>>(k.part, cgs_blocks<T>(n, cgs_vec<T>(n, b, b)), k.ad);
-    dscale_kernel<T><<<vblocks(n), 256, 0, st>>>(n, b, &k.ad->scale, k.V);
+    if ((rc = gs_step<T>(k, 0, n, b, k.V, 0, k.ad, false, st))) return rc;
   }
   for (int j = 0; j < m; ++j) {
     T* vj = k.V + (size_t)j * n;
     T* zj = k.Z + (size_t)j * n;
     if ((rc = precond_t<T>(s, vj, zj, st))) return rc;
     if ((rc = apply_t<T>(s, zj, k.w, st))) return rc;
-    const int nv = j + 1;
     ProfScope ps(FV_K_CGS + lvl, st);
-    CgsFuse f;
-    f.ticket = k.ticket;
-    f.out = k.h;
-    cgs_launch<T>(nv, n, k.V, nullptr, k.w, k.part, 0, st, f);
-    if (once) {  // one pass: w -= V h1 with the norm; the second coefficients stay zero
-      f.out = k.h + 2 * KMAX, f.ad = k.ad, f.gj = j, f.hg = k.h;
-      cgs_launch<T>(nv, n, k.V, k.h, k.w, k.part, 2, st, f);
-    } else {
-      f.out = k.h + KMAX;
-      cgs_launch<T>(nv, n, k.V, k.h, k.w, k.part, 1, st, f);
-      f.out = k.h + 2 * KMAX, f.ad = k.ad, f.gj = j, f.hg = k.h;
-      cgs_launch<T>(nv, n, k.V, k.h + KMAX, k.w, k.part, 2, st, f);
-    }
-    if (j + 1 < m) dscale_kernel<T><<<vblocks(n), 256, 0, st>>>(n, k.w, &k.ad->scale, k.V + (size_t)(j + 1) * n);
+    if ((rc = gs_step<T>(k, j + 1, n, k.w, j + 1 < m ? k.V + (size_t)(j + 1) * n : nullptr, once ? 1 : 2, k.ad, j + 1 == m, st)))
+      return rc;
   }
   ProfScope ps(FV_K_VEC, st);
-  lsq_kernel<<<1, 32, 0, st>>>(m, k.ad);
   dupdate_dispatch<T>(m, vblocks(n), n, k.Z, k.ad->y, x, st, std::make_integer_sequence<int, KMAX>{});
   FV_CUDA(cudaGetLastError());
   return FV_OK;
@@ -646,13 +1031,12 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
   if ((rc = apply_t<T>(s, x, k.r, st))) return rc;
   if ((rc = axpby_t<T>(n, 1.0, b, -1.0, k.r, k.r, st))) return rc;
   double beta;
-  if ((rc = norm2<T>(k, n, k.r, st, &beta))) return rc;
+  if ((rc = norm2<T>(k, n, k.r, k.V, st, &beta))) return rc;
   const double r0 = beta, target = std::max(o->atol, o->rtol * r0);
   int its = 0;
   bool nan = !std::isfinite(beta);
   std::vector<double> H((m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
   while (!nan && beta > target && its < o->max_it) {
-    if ((rc = axpby_t<T>(n, 1.0 / beta, k.r, 0.0, nullptr, k.V, st))) return rc;
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int j = 0;
@@ -665,14 +1049,8 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
       const int nv = j + 1;
       {
         ProfScope ps(FV_K_CGS + lvl, st);
-        CgsFuse f;
-        f.ticket = k.ticket;
-        f.out = k.h;
-        cgs_launch<T>(nv, n, k.V, nullptr, k.w, k.part, 0, st, f);
-        f.out = k.h + KMAX;
-        cgs_launch<T>(nv, n, k.V, k.h, k.w, k.part, 1, st, f);
-        f.out = k.h + 2 * KMAX;
-        cgs_launch<T>(nv, n, k.V, k.h + KMAX, k.w, k.part, 2, st, f);
+        // with the next basis vector (k.V holds m + 1)
+        if ((rc = gs_step<T>(k, nv, n, k.w, k.V + (size_t)(j + 1) * n, 2, nullptr, false, st))) return rc;
       }
       FV_CUDA(cudaGetLastError());
       FV_CUDA(cudaMemcpyAsync(k.hhost, k.h, 3 * KMAX * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -703,7 +1081,6 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
         ++j;
         break;
       }
-      if ((rc = axpby_t<T>(n, 1.0 / hn, k.w, 0.0, nullptr, k.V + (size_t)(j + 1) * n, st))) return rc;
     }
     const int kk = std::min(j, m);
     if (!nan) {
@@ -720,10 +1097,11 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
     }
     if ((rc = apply_t<T>(s, x, k.r, st))) return rc;
     if ((rc = axpby_t<T>(n, 1.0, b, -1.0, k.r, k.r, st))) return rc;
-    if ((rc = norm2<T>(k, n, k.r, st, &beta))) return rc;
+    if ((rc = norm2<T>(k, n, k.r, k.V, st, &beta))) return rc;
     if (!std::isfinite(beta)) nan = true;
     if (breakdown) break;
   }
+  if (*(volatile int*)k.err) return *k.err = 0, set_error("fv_gmres_solve: a grid barrier ran out"), FV_ECUDA;
   if (sweep_failed(s)) return set_error("fv_gmres_solve: a wait of the subdomain sweeps ran out"), FV_ECUDA;
   const bool conv = !nan && beta <= target;
   if (stats) {
