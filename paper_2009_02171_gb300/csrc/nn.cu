@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
 #include "../../include/fv_net.h"
@@ -38,7 +39,6 @@ constexpr int BZ = 4, BY = 4, BX = 8;  // output brick of one convolution CTA (1
 constexpr int HY = BY + 2, HX = BX + 2, HV = (BZ + 2) * HY * HX;
 constexpr int CONV_THREADS = 128;
 constexpr int MAX_CIN = 64;            // widest convolution input (2C, C <= 32)
-constexpr int WK = 64;                 // voxels per weight-gradient chunk
 constexpr int RED_THREADS = 256;
 
 enum { EPI_RELU = 0, EPI_RAW = 1, EPI_FINAL = 2 };
@@ -139,116 +139,156 @@ __device__ __forceinline__ void cp16(void* dst, const void* src, const void* any
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src ? src : any), "r"(n) : "memory");
 }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // NT: output channels / 8 (n tiles), CIN: input channels (a.cin); both fixed at compile time, so the
-// staging index arithmetic reduces to shifts and the tap and channel loops unroll
-template <int NT, int CIN>
-__global__ void __launch_bounds__(CONV_THREADS) conv_kernel(ConvArgs a) {
+// staging index arithmetic reduces to shifts and the tap and channel loops unroll.
+// A CTA stages the weights once and walks over bricks (blockIdx.x, + gridDim.x, ...), with STAGES halo buffers: the
+// next brick's halo is copied while this one is multiplied.  Staging 20 KB of weights for each 128-voxel brick
+// bound the one-brick CTAs (level 0, C = 16, 8 samples of 6x32^3: 182 -> 133 us a convolution).
+template <int NT, int CIN, int STAGES>
+__global__ void __launch_bounds__(CONV_THREADS) conv_kernel(const __grid_constant__ ConvArgs a, int bricks) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  bf16* hs = reinterpret_cast<bf16*>(smem_raw);
   constexpr int cs = CIN + 8;
+  bf16* ws = reinterpret_cast<bf16*>(smem_raw);
+  bf16* hs0 = ws + 27 * NT * 8 * cs;
   const int nbx = (a.On + BX - 1) / BX, nby = (a.On + BY - 1) / BY, nbz = (a.L.Z + BZ - 1) / BZ;
-  int blk = blockIdx.x;
-  const int bx = blk % nbx;
-  blk /= nbx;
-  const int by = blk % nby;
-  blk /= nby;
-  const int bz = blk % nbz;
-  const int p = blk / nbz;
-  const int x0 = a.o0 + bx * BX, y0 = a.o0 + by * BY, z0 = bz * BZ;  // padded coordinates of the brick origin
-
   constexpr int qn = CIN >> 3;
-  for (int it = threadIdx.x; it < HV * qn; it += CONV_THREADS) {
-    const int hv = it / qn, q = it - hv * qn;
-    const int hx = hv % HX, hy = (hv / HX) % HY, hz = hv / (HX * HY);
-    cp16(hs + hv * cs + q * 8,
-         src_in(a.s0, a.c0, a.s1, a.c1, q, p, z0 - 1 + hz, y0 - 1 + hy, x0 - 1 + hx, a.L, a.i0, a.i1), a.w);
+  // brick blk: panel and origin (padded coordinates)
+  auto origin = [&](int blk, int& p, int& x0, int& y0, int& z0) {
+    x0 = a.o0 + blk % nbx * BX;
+    blk /= nbx;
+    y0 = a.o0 + blk % nby * BY;
+    blk /= nby;
+    z0 = blk % nbz * BZ;
+    p = blk / nbz;
+  };
+  // this thread's copies of a halo: position in the halo, packed once (the divisions are not repeated per brick)
+  constexpr int COPIES = (HV * qn + CONV_THREADS - 1) / CONV_THREADS;
+  int at[COPIES];
+#pragma unroll
+  for (int u = 0; u < COPIES; ++u) {
+    const int hv = (threadIdx.x + u * CONV_THREADS) / qn;
+    at[u] = hv % HX | (hv / HX) % HY << 8 | hv / (HX * HY) << 16;
   }
-  // all 27 taps' weights, rows (tap, n) of cin values, staged once: the tap loop then reads the B
-  // fragments from shared memory instead of waiting on global loads
-  bf16* ws = hs + HV * cs;
+  auto stage = [&](int blk, bf16* hs) {
+    int p, x0, y0, z0;
+    origin(blk, p, x0, y0, z0);
+#pragma unroll
+    for (int u = 0; u < COPIES; ++u) {
+      const int it = threadIdx.x + u * CONV_THREADS, hv = it / qn, q = it - hv * qn;
+      if (it >= HV * qn) break;
+      cp16(hs + hv * cs + q * 8,
+           src_in(a.s0, a.c0, a.s1, a.c1, q, p, z0 - 1 + (at[u] >> 16), y0 - 1 + (at[u] >> 8 & 255), x0 - 1 + (at[u] & 255),
+                  a.L, a.i0, a.i1),
+           a.w);
+    }
+  };
+  // all 27 taps' weights, rows (tap, n) of cin values
   for (int it = threadIdx.x; it < 27 * NT * 8 * qn; it += CONV_THREADS) {
     const int row = it / qn, q = it - row * qn;
     cp16(ws + row * cs + q * 8, a.w + (size_t)row * CIN + q * 8, a.w);
   }
-  cp_wait_all();
-  __syncthreads();
+  stage(blockIdx.x, hs0);
+  cp_commit();
+  int turn = 0;
+  for (int blk = blockIdx.x; blk < bricks; blk += gridDim.x, turn ^= STAGES - 1) {
+    bf16* hs = hs0 + turn * HV * cs;
+    const int next = blk + gridDim.x;
+    if (STAGES == 2 && next < bricks) {
+      stage(next, hs0 + (turn ^ 1) * HV * cs);
+      cp_commit();
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    int p, x0, y0, z0;
+    origin(blk, p, x0, y0, z0);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float acc[2][NT][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float acc[2][NT][4];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+      for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
+        for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
 
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(hs);
-  // A rows: lane & 15 = row of the m16 tile (y offset row >> 3, x offset row & 7), lane >> 4 = k half
-  const int r = lane & 15, kh = lane >> 4;
-  int hv0[2];
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(hs);
+    // A rows: lane & 15 = row of the m16 tile (y offset row >> 3, x offset row & 7), lane >> 4 = k half
+    const int r = lane & 15, kh = lane >> 4;
+    int hv0[2];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt) hv0[mt] = (warp * HY + 2 * mt + (r >> 3)) * HX + (r & 7);
-  // B rows: lanes 0-7 / 8-15 give n-tile 2j's rows at k halves 0 / 1, lanes 16-31 n-tile 2j + 1's
-  const uint32_t wbase = sbase + (uint32_t)(HV * cs * 2);
-  const int brow = ((lane >> 4) * 8 + (lane & 7)), bk = ((lane >> 3) & 1) * 8;
+    for (int mt = 0; mt < 2; ++mt) hv0[mt] = (warp * HY + 2 * mt + (r >> 3)) * HX + (r & 7);
+    // B rows: lanes 0-7 / 8-15 give n-tile 2j's rows at k halves 0 / 1, lanes 16-31 n-tile 2j + 1's
+    const uint32_t wbase = (uint32_t)__cvta_generic_to_shared(ws);
+    const int brow = ((lane >> 4) * 8 + (lane & 7)), bk = ((lane >> 3) & 1) * 8;
 #pragma unroll
-  for (int tap = 0; tap < 27; ++tap) {
-    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-    const int toff = (dz * HY + dy) * HX + dx;
+    for (int tap = 0; tap < 27; ++tap) {
+      const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
+      const int toff = (dz * HY + dy) * HX + dx;
 #pragma unroll
-    for (int kc = 0; kc < CIN; kc += 16) {
-      uint32_t af[2][4];
+      for (int kc = 0; kc < CIN; kc += 16) {
+        uint32_t af[2][4];
 #pragma unroll
-      for (int mt = 0; mt < 2; ++mt) ldsm4(sbase + (uint32_t)(((hv0[mt] + toff) * cs + kc + kh * 8) * 2), af[mt]);
+        for (int mt = 0; mt < 2; ++mt) ldsm4(sbase + (uint32_t)(((hv0[mt] + toff) * cs + kc + kh * 8) * 2), af[mt]);
 #pragma unroll
-      for (int np = 0; np < (NT + 1) / 2; ++np) {
-        uint32_t bf[4];
-        const int row = tap * NT * 8 + np * 16 + (NT == 1 ? (lane & 7) : brow);
-        ldsm4(wbase + (uint32_t)((row * cs + kc + bk) * 2), bf);
+        for (int np = 0; np < (NT + 1) / 2; ++np) {
+          uint32_t bf[4];
+          const int row = tap * NT * 8 + np * 16 + (NT == 1 ? (lane & 7) : brow);
+          ldsm4(wbase + (uint32_t)((row * cs + kc + bk) * 2), bf);
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          mma16816(acc[mt][2 * np], af[mt], bf[0], bf[1]);
-          if (2 * np + 1 < NT) mma16816(acc[mt][2 * np + 1], af[mt], bf[2], bf[3]);
+          for (int mt = 0; mt < 2; ++mt) {
+            mma16816(acc[mt][2 * np], af[mt], bf[0], bf[1]);
+            if (2 * np + 1 < NT) mma16816(acc[mt][2 * np + 1], af[mt], bf[2], bf[3]);
+          }
         }
       }
+    }
+
+    // epilogue: accumulator e of tile (mt, nt): row (lane >> 2) + 8 (e >> 1), column nt*8 + (lane & 3)*2 + (e & 1)
+    const int z = z0 + warp;
+    const int Yp = a.L.Y + 2, Xp = a.L.X + 2;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = (lane >> 2) + 8 * h;
+        const int y = y0 + 2 * mt + (row >> 3), x = x0 + (row & 7);
+        if (z >= a.L.Z || y >= a.o0 + a.On || x >= a.o0 + a.On) continue;
+        const long long v = (((long long)p * a.L.Z + z) * Yp + y) * Xp + x;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          const int col = nt * 8 + (lane & 3) * 2;
+          float u0 = acc[mt][nt][2 * h], u1 = acc[mt][nt][2 * h + 1];
+          if (a.mode == EPI_FINAL) {  // interior cell index (y, x >= 1 here)
+            const long long c = (((long long)p * a.L.Z + z) * a.L.Y + (y - 1)) * a.L.X + (x - 1);
+            if (col < a.cout) a.y[c * a.cout + col] = u0 + a.bias[col];
+            if (col + 1 < a.cout) a.y[c * a.cout + col + 1] = u1 + a.bias[col + 1];
+            continue;
+          }
+          if (col >= a.cout) continue;
+          if (a.mode == EPI_RELU) {
+            u0 = fmaxf(u0 + a.bias[col], 0.f);
+            u1 = fmaxf(u1 + a.bias[col + 1], 0.f);
+          }
+          const __nv_bfloat162 o = __floats2bfloat162_rn(u0, u1);
+          *reinterpret_cast<__nv_bfloat162*>(a.out + v * a.cout + col) = o;
+          if (a.ring)  // the cell is the source of the ring voxel across each panel edge it touches
+            ring_targets(a.H, a.L.Y, a.L.Z, p, z, y - 1, x - 1, [&](long long rv) {
+              *reinterpret_cast<__nv_bfloat162*>(a.out + rv * a.cout + col) = o;
+            });
+        }
+      }
+    __syncthreads();  // the halo buffer is free
+    if (STAGES == 1 && next < bricks) {
+      stage(next, hs0);
+      cp_commit();
     }
   }
-
-  // epilogue: accumulator e of tile (mt, nt): row (lane >> 2) + 8 (e >> 1), column nt*8 + (lane & 3)*2 + (e & 1)
-  const int z = z0 + warp;
-  const int Yp = a.L.Y + 2, Xp = a.L.X + 2;
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int row = (lane >> 2) + 8 * h;
-      const int y = y0 + 2 * mt + (row >> 3), x = x0 + (row & 7);
-      if (z >= a.L.Z || y >= a.o0 + a.On || x >= a.o0 + a.On) continue;
-      const long long v = (((long long)p * a.L.Z + z) * Yp + y) * Xp + x;
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int col = nt * 8 + (lane & 3) * 2;
-        float u0 = acc[mt][nt][2 * h], u1 = acc[mt][nt][2 * h + 1];
-        if (a.mode == EPI_FINAL) {  // interior cell index (y, x >= 1 here)
-          const long long c = (((long long)p * a.L.Z + z) * a.L.Y + (y - 1)) * a.L.X + (x - 1);
-          if (col < a.cout) a.y[c * a.cout + col] = u0 + a.bias[col];
-          if (col + 1 < a.cout) a.y[c * a.cout + col + 1] = u1 + a.bias[col + 1];
-          continue;
-        }
-        if (col >= a.cout) continue;
-        if (a.mode == EPI_RELU) {
-          u0 = fmaxf(u0 + a.bias[col], 0.f);
-          u1 = fmaxf(u1 + a.bias[col + 1], 0.f);
-        }
-        const __nv_bfloat162 o = __floats2bfloat162_rn(u0, u1);
-        *reinterpret_cast<__nv_bfloat162*>(a.out + v * a.cout + col) = o;
-        if (a.ring)  // the cell is the source of the ring voxel across each panel edge it touches
-          ring_targets(a.H, a.L.Y, a.L.Z, p, z, y - 1, x - 1, [&](long long rv) {
-            *reinterpret_cast<__nv_bfloat162*>(a.out + rv * a.cout + col) = o;
-          });
-      }
-    }
 }
 
 // Adjoint of the ring fill on a gradient over the whole padded plane: every edge cell gets
@@ -289,15 +329,25 @@ __global__ void halo_adjoint_kernel(bf16* __restrict__ g, int C, int P, Lvl L, H
   }
 }
 
-// g <- g * (a > 0) on interior cells, 0 on the ring (padded tensors of C channels)
-__global__ void mask_kernel(bf16* __restrict__ g, const bf16* __restrict__ a, int C, int P, Lvl L) {
-  const long long total = L.vox(P) * C;
-  const int Yp = L.Y + 2, Xp = L.X + 2;
+// out = g * (a > 0) on interior cells, 0 on the ring (padded tensors of C channels; out may be g): eight channels a
+// thread, the copy of g into out fused with the mask
+__global__ void mask_kernel(const bf16* g, const bf16* __restrict__ a, bf16* out, int C, int P, Lvl L) {
+  const int qn = C / 8, Yp = L.Y + 2, Xp = L.X + 2;
+  const long long total = L.vox(P) * qn;
   for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < total; it += (long long)gridDim.x * blockDim.x) {
-    const long long v = it / C;
-    const int x = (int)(v % Xp), y = (int)((v / Xp) % Yp);
-    const bool in = x >= 1 && x <= L.X && y >= 1 && y <= L.Y;
-    g[it] = (in && __bfloat162float(a[it]) > 0.f) ? g[it] : __float2bfloat16_rn(0.f);
+    const long long v = it / qn;
+    const unsigned r = (unsigned)(v % ((long long)Xp * Yp));
+    const int x = r % Xp, y = r / Xp;
+    uint4 o = make_uint4(0, 0, 0, 0);
+    if (x >= 1 && x <= L.X && y >= 1 && y <= L.Y) {
+      const uint4 av = reinterpret_cast<const uint4*>(a)[it], gv = reinterpret_cast<const uint4*>(g)[it];
+      const bf16 *ah = reinterpret_cast<const bf16*>(&av), *gh = reinterpret_cast<const bf16*>(&gv);
+      bf16* oh = reinterpret_cast<bf16*>(&o);
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (__bfloat162float(ah[c]) > 0.f) oh[c] = gh[c];
+    }
+    reinterpret_cast<uint4*>(out)[it] = o;
   }
 }
 
@@ -361,153 +411,211 @@ __global__ void pool_kernel(const bf16* __restrict__ a, bf16* __restrict__ out, 
 __global__ void split_kernel(const bf16* __restrict__ gcat, bf16* __restrict__ gE, bf16* __restrict__ gnext,
                              const bf16* __restrict__ mask, int C, int P, Lvl Lc) {
   const Lvl L{Lc.Z * 2, Lc.Y * 2, Lc.X * 2};
-  const long long total = Lc.cells(P) * C;
+  const int qn = C / 8;
+  const long long total = Lc.cells(P) * qn;
   for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < total; it += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(it % C);
-    const long long cell = it / C;
-    const int x = (int)(cell % Lc.X), y = (int)((cell / Lc.X) % Lc.Y);
-    const long long pz = cell / ((long long)Lc.X * Lc.Y);
+    const int q = (int)(it % qn);
+    const long long pv = padded(it / qn, Lc), cell = it / qn, pz = cell / (Lc.X * Lc.Y);
+    const int r = (int)(cell - pz * (Lc.X * Lc.Y)), x = r % Lc.X, y = r / Lc.X;
     const int z = (int)(pz % Lc.Z);
     const long long p = pz / Lc.Z;
-    float s = 0.f;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     for (int k = 0; k < 8; ++k) {
       const long long v = (((p * L.Z + 2 * z + (k >> 2)) * (L.Y + 2) + 2 * y + ((k >> 1) & 1) + 1) * (L.X + 2) + 2 * x +
                            (k & 1) + 1);
-      gE[v * C + c] = gcat[v * 2 * C + c];
-      s += __bfloat162float(gcat[v * 2 * C + C + c]);
+      const uint4* src = reinterpret_cast<const uint4*>(gcat + v * 2 * C) + q;
+      reinterpret_cast<uint4*>(gE + v * C)[q] = src[0];
+      const uint4 u = src[qn];
+      const bf16* h = reinterpret_cast<const bf16*>(&u);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) s[c] += __bfloat162float(h[c]);
     }
-    const long long pv = padded(cell, Lc) * C + c;
-    if (mask && !(__bfloat162float(mask[pv]) > 0.f)) s = 0.f;
-    gnext[pv] = __float2bfloat16_rn(s);
+    uint4 o, m = make_uint4(0, 0, 0, 0);
+    if (mask) m = reinterpret_cast<const uint4*>(mask + pv * C)[q];
+    const bf16* mh = reinterpret_cast<const bf16*>(&m);
+    bf16* oh = reinterpret_cast<bf16*>(&o);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) oh[c] = __float2bfloat16_rn(mask && !(__bfloat162float(mh[c]) > 0.f) ? 0.f : s[c]);
+    reinterpret_cast<uint4*>(gnext + pv * C)[q] = o;
   }
 }
 
 // encoder backward through the pooling: gE[child] += g[parent] / 8 (interiors; Lc = parent level)
 __global__ void unpool_add_kernel(const bf16* __restrict__ g, bf16* __restrict__ gE, int C, int P, Lvl Lc) {
   const Lvl L{Lc.Z * 2, Lc.Y * 2, Lc.X * 2};
-  const long long total = L.cells(P) * C;
+  const int qn = C / 8;
+  const long long total = L.cells(P) * qn;
   for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < total; it += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(it % C);
-    const long long cell = it / C;
-    const int x = (int)(cell % L.X), y = (int)((cell / L.X) % L.Y);
-    const long long pz = cell / ((long long)L.X * L.Y);
+    const int q = (int)(it % qn);
+    const long long cell = it / qn, pz = cell / (L.X * L.Y);
+    const int r = (int)(cell - pz * (L.X * L.Y)), x = r % L.X, y = r / L.X;
     const int z = (int)(pz % L.Z);
     const long long p = pz / L.Z;
     const long long pc = ((p * Lc.Z + z / 2) * Lc.Y + y / 2) * Lc.X + x / 2;
-    const long long v = padded(cell, L) * C + c;
-    gE[v] = __float2bfloat16_rn(__bfloat162float(gE[v]) + 0.125f * __bfloat162float(g[padded(pc, Lc) * C + c]));
+    uint4* dst = reinterpret_cast<uint4*>(gE + padded(cell, L) * C) + q;
+    uint4 e = *dst;
+    const uint4 u = reinterpret_cast<const uint4*>(g + padded(pc, Lc) * C)[q];
+    bf16* eh = reinterpret_cast<bf16*>(&e);
+    const bf16* uh = reinterpret_cast<const bf16*>(&u);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) eh[c] = __float2bfloat16_rn(__bfloat162float(eh[c]) + 0.125f * __bfloat162float(uh[c]));
+    *dst = e;
   }
 }
 
 // Weight gradient of one convolution: gw[co][ci][tap] = sum over interior output cells v of
-// in[v + tap offset][ci] * g[v][co].  CTA (chunk group, tap); warp pairs (16 input channels) x
-// (16 output channels) accumulate over WK-cell chunks; each CTA stores its partial tile and
-// wsum_kernel adds the groups' tiles in a fixed order (bitwise reproducible training).
+// in[v + tap offset][ci] * g[v][co].  CTA (group of voxel chunks, dz, 32 input channels): it walks over its chunks of
+// WK consecutive cells with the three (eta) rows of input around every row of cells in shared memory, so a staged
+// voxel serves the nine taps of its dz, one a warp: a tap is an offset of the lanes' ldmatrix addresses.  Staging
+// input and gradient again for every tap was 10.9 of the 15.0 ms of a gradient (C = 16, 8 samples of 6x32^3; 6.1 ms
+// now).  What is left is each chunk's copies, barrier and a chain of four multiply-accumulates.  The order of a sum (chunks of a group, 16 cells a multiply-accumulate, then the groups in order) depends on the cell
+// count alone: training is bitwise reproducible.
 struct WGradArgs {
   const bf16* s0;
   const bf16* s1;
   const bf16* g;
-  float* part;  // [CTA group][tap][co][ci] partial sums (summed in a fixed order: deterministic)
-  int c0, c1, cin, gc, ci, co;
-  int P;
+  float* part;  // [group][tap][co][ci] partial sums
+  int c0, c1, ci, co;
+  int P, pw, nr;  // voxels of a staged row, rows of cells a chunk may touch
   Lvl L;
   long long chunks_per_cta;
 };
 
-constexpr int WG_PAIRS = 4;     // (16 x 16) output tiles per warp: cin/16 * gc/16 <= 16
+constexpr int WK = 64;          // cells a chunk
 constexpr int WG_GROUPS = 48;   // voxel-range groups of the weight gradient (partial tiles)
 constexpr int BG_BLOCKS = 640;  // blocks of the bias gradient (partial sums)
 constexpr int SS_BLOCKS = 320;  // blocks per sample of the sum of squares
+constexpr int WG_THREADS = 9 * 32;
 
-__global__ void __launch_bounds__(CONV_THREADS) wgrad_kernel(WGradArgs a) {
+template <int CIN, int GC, int STAGES>
+__global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const __grid_constant__ WGradArgs a) {
+  constexpr int cs = CIN + 8, gsn = GC + 8, MT = CIN / 16, NT2 = GC / 16, qx = CIN / 8, qg = GC / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int xsn = a.cin + 8, gsn = a.gc + 8;
-  bf16* xs = reinterpret_cast<bf16*>(smem_raw);
-  bf16* gs = xs + WK * xsn;
-  const int tap = blockIdx.y;
-  const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-  const long long V = a.L.cells(a.P);
-  const long long nchunk = (V + WK - 1) / WK;
+  bf16* const buf = reinterpret_cast<bf16*>(smem_raw);
+  const int X = a.L.X, rows = a.nr * 3 * a.pw, STG = rows * cs + WK * gsn;
+  const long long V = a.L.cells(a.P), nchunk = (V + WK - 1) / WK;
   const long long c_begin = blockIdx.x * a.chunks_per_cta;
   const long long c_end = nchunk < c_begin + a.chunks_per_cta ? nchunk : c_begin + a.chunks_per_cta;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n16 = a.gc >> 4, pairs = (a.cin >> 4) * n16;
-  float acc[WG_PAIRS][2][4];
+  const int dz = (int)blockIdx.y - 1, qoff = blockIdx.z * qx;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q4 = lane >> 3, i8 = lane & 7;
+  const int dy = warp / 3, dx = warp % 3;  // this warp's tap, 0 .. 2
+  const bool wide = X > WK;                // a chunk touches at most two rows: only its part of the first is staged
+  // this thread's first copies of a chunk, decoded once: x within the row, dy, row of cells
+  constexpr int KEEP = 4;
+  auto decode = [&](int it) {
+    const int vx = it / qx, t = vx / a.pw;
+    return (vx - t * a.pw) | t % 3 << 8 | t / 3 << 16;
+  };
+  int at0[KEEP];
 #pragma unroll
-  for (int i = 0; i < WG_PAIRS; ++i)
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][h][e] = 0.f;
-  const uint32_t xbase = (uint32_t)__cvta_generic_to_shared(xs), gbase = (uint32_t)__cvta_generic_to_shared(gs);
-  const int q = lane >> 3, i8 = lane & 7;
-  const int qx = a.cin >> 3, qg = a.gc >> 3;
-  for (long long ch = c_begin; ch < c_end; ++ch) {
-    __syncthreads();
-    for (int it = threadIdx.x; it < WK * qx; it += CONV_THREADS) {
-      const int k = it / qx, qq = it - k * qx;
-      const long long v = ch * WK + k;
-      const bf16* src = nullptr;
-      if (v < V) {
-        long long t = v;
-        const int x = (int)(t % a.L.X);
-        t /= a.L.X;
-        const int y = (int)(t % a.L.Y);
-        t /= a.L.Y;
-        const int z = (int)(t % a.L.Z);
-        const int p = (int)(t / a.L.Z);
-        src = src_in(a.s0, a.c0, a.s1, a.c1, qq, p, z + dz, y + 1 + dy, x + 1 + dx, a.L, 0, a.L.Y + 2);
+  for (int u = 0; u < KEEP; ++u) at0[u] = decode(threadIdx.x + u * WG_THREADS);
+  auto stage = [&](long long ch, bf16* xs) {
+    const long long v0 = ch * WK, r0 = v0 / X, v1 = (v0 + WK < V ? v0 + WK : V) - 1;
+    const int x00 = wide ? (int)(v0 - r0 * X) : 0, n = (int)(v1 / X - r0 + 1) * 3 * a.pw * qx;
+    const unsigned pz0 = (unsigned)r0 / a.L.Y;
+    const int y0 = (int)((unsigned)r0 - pz0 * a.L.Y), p0 = (int)(pz0 / a.L.Z), z0 = (int)(pz0 - p0 * a.L.Z);
+    auto copy = [&](int it, int d) {
+      const int vx = it / qx, q = it - vx * qx, i = d >> 16;
+      int y = y0 + i, z = z0, p = p0;
+      while (y >= a.L.Y) {
+        y -= a.L.Y;
+        if (++z == a.L.Z) z = 0, ++p;
       }
-      cp16(xs + k * xsn + qq * 8, src, a.g);
+      cp16(xs + vx * cs + q * 8,
+           src_in(a.s0, a.c0, a.s1, a.c1, qoff + q, p, z + dz, y + (d >> 8 & 3), (d & 255) + (i == 0 ? x00 : 0), a.L, 0, a.L.Y + 2),
+           a.g);
+    };
+#pragma unroll
+    for (int u = 0; u < KEEP; ++u)
+      if ((int)threadIdx.x + u * WG_THREADS < n) copy(threadIdx.x + u * WG_THREADS, at0[u]);
+    for (int it = threadIdx.x + KEEP * WG_THREADS; it < n; it += WG_THREADS) copy(it, decode(it));
+    bf16* gs = xs + rows * cs;
+    for (int it = threadIdx.x; it < WK * qg; it += WG_THREADS) {
+      const int k = it / qg, q = it - k * qg;
+      cp16(gs + k * gsn + q * 8, v0 + k < V ? a.g + padded(v0 + k, a.L) * GC + q * 8 : nullptr, a.g);
     }
-    for (int it = threadIdx.x; it < WK * qg; it += CONV_THREADS) {
-      const int k = it / qg, qq = it - k * qg;
-      const long long v = ch * WK + k;
-      cp16(gs + k * gsn + qq * 8, v < V ? a.g + padded(v, a.L) * a.gc + qq * 8 : nullptr, a.g);
-    }
-    cp_wait_all();
-    __syncthreads();
+  };
+  float acc[MT][NT2][2][4];
+#pragma unroll
+  for (int e = 0; e < MT * NT2 * 8; ++e) (&acc[0][0][0][0])[e] = 0.f;
+  // staged voxel of this lane's A row in each of the chunk's four 16-cell steps
+  int at[WK / 16];
+  const bool fixed = WK % X == 0;  // chunks start rows: the same in every chunk
+  auto rows_of = [&](long long ch) {
+    const long long v0 = ch * WK, r0 = v0 / X;
+    const int x00 = wide ? (int)(v0 - r0 * X) : 0;
 #pragma unroll
     for (int kk = 0; kk < WK / 16; ++kk) {
+      long long v = v0 + kk * 16 + (q4 >> 1) * 8 + i8;
+      if (v >= V) v = V - 1;  // past the end the gradient is zero: any staged voxel
+      const int r = (int)(v / X - r0), x = (int)(v % X);
+      at[kk] = (r * 3 + dy) * a.pw + x + dx - (r == 0 ? x00 : 0);
+    }
+  };
+  // STAGES - 1 chunks ahead, one commit group a chunk; with one buffer a chunk is copied when the last is done
+  constexpr int AHEAD = STAGES > 1 ? STAGES - 1 : 1;
 #pragma unroll
-      for (int i = 0; i < WG_PAIRS; ++i) {
-        const int pr = warp + 4 * i;
-        if (pr >= pairs) continue;
-        const int mt = pr / n16, nt = pr - mt * n16;
-        uint32_t af[4], bf[4];
-        // A = in^T (m = input channel, k = voxel): matrix q covers voxels (q >> 1) * 8, channels (q & 1) * 8
-        ldsm4t(xbase + (uint32_t)(((kk * 16 + (q >> 1) * 8 + i8) * xsn + mt * 16 + (q & 1) * 8) * 2), af);
-        // B = g (k = voxel, n = output channel): matrix q covers voxels (q & 1) * 8, channels (q >> 1) * 8
-        ldsm4t(gbase + (uint32_t)(((kk * 16 + (q & 1) * 8 + i8) * gsn + nt * 16 + (q >> 1) * 8) * 2), bf);
-        mma16816(acc[i][0], af, bf[0], bf[1]);
-        mma16816(acc[i][1], af, bf[2], bf[3]);
+  for (int u = 0; u < AHEAD; ++u) {
+    if (c_begin + u < c_end) stage(c_begin + u, buf + u * STG);
+    cp_commit();
+  }
+  int turn = 0;
+  for (long long ch = c_begin; ch < c_end; ++ch, turn = turn + 1 == STAGES ? 0 : turn + 1) {
+    if (ch == c_begin || !fixed || ch + 1 == nchunk) rows_of(ch);
+    cp_wait<AHEAD - 1>();
+    __syncthreads();  // chunk ch has landed, the buffer of chunk ch - 1 is free
+    if (STAGES > 1) {
+      if (ch + AHEAD < c_end) stage(ch + AHEAD, buf + (turn == 0 ? STAGES - 1 : turn - 1) * STG);
+      cp_commit();
+    }
+    const uint32_t xb = (uint32_t)__cvta_generic_to_shared(buf + turn * STG), gb = xb + (uint32_t)(rows * cs * 2);
+#pragma unroll
+    for (int kk = 0; kk < WK / 16; ++kk) {
+      uint32_t bf[NT2][4];
+#pragma unroll
+      for (int nt = 0; nt < NT2; ++nt)  // B = g: matrix q4 covers cells (q4 & 1) * 8, channels (q4 >> 1) * 8
+        ldsm4t(gb + (uint32_t)(((kk * 16 + (q4 & 1) * 8 + i8) * gsn + nt * 16 + (q4 >> 1) * 8) * 2), bf[nt]);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        uint32_t af[4];  // A = in^T: matrix q4 covers cells (q4 >> 1) * 8, channels (q4 & 1) * 8
+        ldsm4t(xb + (uint32_t)((at[kk] * cs + mt * 16 + (q4 & 1) * 8) * 2), af);
+#pragma unroll
+        for (int nt = 0; nt < NT2; ++nt) {
+          mma16816(acc[mt][nt][0], af, bf[nt][0], bf[nt][1]);
+          mma16816(acc[mt][nt][1], af, bf[nt][2], bf[nt][3]);
+        }
       }
     }
+    if (STAGES == 1) {
+      __syncthreads();
+      if (ch + 1 < c_end) stage(ch + 1, buf);
+      cp_commit();
+    }
   }
+  const int tap = blockIdx.y * 9 + warp;
 #pragma unroll
-  for (int i = 0; i < WG_PAIRS; ++i) {
-    const int pr = warp + 4 * i;
-    if (pr >= pairs) continue;
-    const int mt = pr / n16, nt = pr - mt * n16;
+  for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int nt = 0; nt < NT2; ++nt)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int m = mt * 16 + (lane >> 2) + 8 * (e >> 1);
-        const int n = nt * 16 + h * 8 + (lane & 3) * 2 + (e & 1);
-        if (m < a.ci && n < a.co) a.part[((long long)blockIdx.x * 27 + tap) * a.ci * a.co + n * a.ci + m] = acc[i][h][e];
-      }
-  }
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int m = blockIdx.z * CIN + mt * 16 + (lane >> 2) + 8 * (e >> 1);
+          const int n = nt * 16 + h * 8 + (lane & 3) * 2 + (e & 1);
+          if (m < a.ci && n < a.co) a.part[((long long)blockIdx.x * 27 + tap) * a.ci * a.co + n * a.ci + m] = acc[mt][nt][h][e];
+        }
 }
 
 // gw[co][ci][tap] = sum over the groups (in order) of the partial tiles
 __global__ void wsum_kernel(const float* __restrict__ part, int groups, int ci, int co, float* __restrict__ gw) {
   const int n = 27 * ci * co;
   for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < n; it += gridDim.x * blockDim.x) {
-    const int tap = it % 27, m = (it / 27) % ci, o = it / (27 * ci);
+    const int m = it % ci, o = it / ci % co, tap = it / (ci * co);
     float s = 0.f;
-    for (int g = 0; g < groups; ++g) s += part[((long long)g * 27 + tap) * ci * co + o * ci + m];
-    gw[it] = s;
+#pragma unroll 16
+    for (int g = 0; g < groups; ++g) s += part[(long long)g * n + it];
+    gw[(o * ci + m) * 27 + tap] = s;
   }
 }
 
@@ -518,8 +626,15 @@ __global__ void bgrad_kernel(const bf16* __restrict__ g, int gc, int co, int P, 
   const int c = threadIdx.x % gc, r = threadIdx.x / gc;
   const long long V = L.cells(P);
   float s = 0.f;
-  for (long long v = (long long)blockIdx.x * rows + r; v < V; v += (long long)gridDim.x * rows)
-    s += __bfloat162float(g[padded(v, L) * gc + c]);
+  // eight loads in flight, added in order
+  const long long step = (long long)gridDim.x * rows;
+  for (long long v = (long long)blockIdx.x * rows + r; v < V; v += 8 * step) {
+    float t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = v + u * step < V ? __bfloat162float(g[padded(v + u * step, L) * gc + c]) : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += t[u];
+  }
   part[threadIdx.x] = s;
   __syncthreads();
   if (threadIdx.x < gc) {
@@ -533,6 +648,7 @@ __global__ void bgrad_kernel(const bf16* __restrict__ g, int gc, int co, int P, 
 __global__ void bsum_kernel(const float* __restrict__ bpart, int blocks, int co, float* __restrict__ gb) {
   if (threadIdx.x >= co) return;
   float s = 0.f;
+#pragma unroll 16
   for (int b = 0; b < blocks; ++b) s += bpart[b * co + threadIdx.x];
   gb[threadIdx.x] = s;
 }
@@ -628,14 +744,14 @@ __global__ void unpack_kernel(const float* __restrict__ y, const double* __restr
 // loss = sum over entries of (y - e/s)^2 (accumulated); gy interior = 2 (y - e/s) / ntot in
 // channels 0, 1 of 16 (the ring of gy stays zero)
 __global__ void loss_kernel(const float* __restrict__ y, const double* __restrict__ e, const double* __restrict__ ss,
-                            long long V1, int nb, Lvl L, double inv_ntot, bf16* __restrict__ gy, double* loss) {
+                            long long V1, Lvl L, double inv_ntot, bf16* __restrict__ gy, double* loss) {
   __shared__ double part[RED_THREADS];
-  const long long n = V1 * nb;
+  const long long b = blockIdx.y;  // one sample a grid row: its scale is computed once a thread
+  const double s2 = ss[b];
+  const double inv = s2 > 0.0 ? sqrt(2.0 * (double)V1 / s2) : 0.0;
   double acc = 0.0;
-  for (long long v = blockIdx.x * (long long)RED_THREADS + threadIdx.x; v < n; v += (long long)gridDim.x * RED_THREADS) {
-    const long long b = v / V1, vl = v - b * V1;
-    const double s2 = ss[b];
-    const double inv = s2 > 0.0 ? sqrt(2.0 * (double)V1 / s2) : 0.0;
+  for (long long vl = blockIdx.x * (long long)RED_THREADS + threadIdx.x; vl < V1; vl += (long long)gridDim.x * RED_THREADS) {
+    const long long v = b * V1 + vl;
     const double d0 = (double)y[2 * v] - e[b * 2 * V1 + vl] * inv;
     const double d1 = (double)y[2 * v + 1] - e[b * 2 * V1 + V1 + vl] * inv;
     acc += d0 * d0 + d1 * d1;
@@ -747,37 +863,49 @@ int dL(const fv_net* n, int l) { return 2 * (n->levels + 1) + (n->levels - 1 - l
 int outL(const fv_net* n) { return 2 * (n->levels + 1) + n->levels; }
 
 template <int NT, int CIN>
-fv_status conv_launch_nt(const ConvArgs& a, int blocks, size_t smem, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    FV_CUDA(cudaFuncSetAttribute(conv_kernel<NT, CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr = true;
-  }
-  conv_kernel<NT, CIN><<<blocks, CONV_THREADS, smem, st>>>(a);
+fv_status conv_launch_nt(const ConvArgs& a, int bricks, cudaStream_t st) {
+  constexpr int wbytes = 27 * NT * 8 * (CIN + 8) * 2, hbytes = HV * (CIN + 8) * 2;
+  // two halo buffers for 16 input channels (four CTAs an SM); wider inputs hold one, for the sake of a third CTA
+  constexpr int STAGES = CIN == 16 ? 2 : 1;
+  constexpr int smem = wbytes + STAGES * hbytes;
+  static std::once_flag once[64];
+  static cudaError_t err[64];
+  static int resident[64];  // CTAs the device holds
+  int dev = 0;
+  FV_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return set_error("fv_net: device ordinal out of range"), FV_EINVAL;
+  std::call_once(once[dev], [&] {
+    int per = 0, sms = 0;
+    err[dev] = cudaFuncSetAttribute(conv_kernel<NT, CIN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (!err[dev]) err[dev] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, conv_kernel<NT, CIN, STAGES>, CONV_THREADS, smem);
+    if (!err[dev]) err[dev] = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    resident[dev] = std::max(1, per * sms);
+  });
+  FV_CUDA(err[dev]);
+  // every CTA the same number of bricks, give or take one
+  const int turns = (bricks + resident[dev] - 1) / resident[dev];
+  conv_kernel<NT, CIN, STAGES><<<(bricks + turns - 1) / turns, CONV_THREADS, smem, st>>>(a, bricks);
   return FV_OK;
 }
 
 template <int NT>
-fv_status conv_launch_cin(const ConvArgs& a, int blocks, size_t smem, cudaStream_t st) {
+fv_status conv_launch_cin(const ConvArgs& a, int bricks, cudaStream_t st) {
   switch (a.cin) {
-    case 16: return conv_launch_nt<NT, 16>(a, blocks, smem, st);
-    case 32: return conv_launch_nt<NT, 32>(a, blocks, smem, st);
-    case 48: return conv_launch_nt<NT, 48>(a, blocks, smem, st);
-    case 64: return conv_launch_nt<NT, 64>(a, blocks, smem, st);
+    case 16: return conv_launch_nt<NT, 16>(a, bricks, st);
+    case 32: return conv_launch_nt<NT, 32>(a, bricks, st);
+    case 64: return conv_launch_nt<NT, 64>(a, bricks, st);
     default: return set_error("fv_net: unsupported input channel count"), FV_EINVAL;
   }
 }
 
 fv_status conv(const ConvArgs& a, cudaStream_t st) {
-  const int blocks = a.P * ((a.L.Z + BZ - 1) / BZ) * ((a.On + BY - 1) / BY) * ((a.On + BX - 1) / BX);
-  const size_t smem = (size_t)(HV + 27 * a.coutN) * (a.cin + 8) * 2;  // halo + the staged weights
-  if (a.cin % 16 || a.c0 % 8 || a.cin > MAX_CIN || a.coutN % 8 || smem > 200 * 1024)
-    return set_error("fv_net: bad convolution shape"), FV_EINVAL;
+  const int bricks = a.P * ((a.L.Z + BZ - 1) / BZ) * ((a.On + BY - 1) / BY) * ((a.On + BX - 1) / BX);
+  if (a.cin % 16 || a.c0 % 8 || a.cin > MAX_CIN || a.coutN % 8) return set_error("fv_net: bad convolution shape"), FV_EINVAL;
   switch (a.coutN / 8) {
-    case 1: return conv_launch_cin<1>(a, blocks, smem, st);
-    case 2: return conv_launch_cin<2>(a, blocks, smem, st);
-    case 4: return conv_launch_cin<4>(a, blocks, smem, st);
-    case 8: return conv_launch_cin<8>(a, blocks, smem, st);
+    case 1: return conv_launch_cin<1>(a, bricks, st);
+    case 2: return conv_launch_cin<2>(a, bricks, st);
+    case 4: return conv_launch_cin<4>(a, bricks, st);
+    case 8: return conv_launch_cin<8>(a, bricks, st);
     default: return set_error("fv_net: unsupported output channel count"), FV_EINVAL;
   }
 }
@@ -798,24 +926,52 @@ ConvArgs bwd_args(const bf16* g, const NetLayer& ly, bf16* out, int P, const Lvl
   return a;
 }
 
+constexpr int WG_SMEM = 220 * 1024;
+
+template <int CIN, int GC, int STAGES>
+fv_status wgrad_launch_n(const WGradArgs& a, int cin, int groups, size_t stage, cudaStream_t st) {
+  static std::once_flag once[64];
+  static cudaError_t err[64];
+  int dev = 0;
+  FV_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return set_error("fv_net: device ordinal out of range"), FV_EINVAL;
+  std::call_once(once[dev], [&] {
+    err[dev] = cudaFuncSetAttribute(wgrad_kernel<CIN, GC, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
+  });
+  FV_CUDA(err[dev]);
+  wgrad_kernel<CIN, GC, STAGES><<<dim3(groups, 3, cin / CIN), WG_THREADS, STAGES * stage, st>>>(a);
+  return FV_OK;
+}
+
+// four buffers where they fit (rows of 4 cells and more), else one: at most 64 rows of 3 x 3 voxels, 57 KB
+template <int CIN, int GC>
+fv_status wgrad_launch(const WGradArgs& a, int cin, int groups, cudaStream_t st) {
+  const size_t stage = ((size_t)a.nr * 3 * a.pw * (CIN + 8) + WK * (GC + 8)) * 2;
+  return 4 * stage <= (size_t)WG_SMEM ? wgrad_launch_n<CIN, GC, 4>(a, cin, groups, stage, st)
+                                      : wgrad_launch_n<CIN, GC, 1>(a, cin, groups, stage, st);
+}
+
 fv_status wgrad(fv_net* n, const bf16* s0, int c0, const bf16* s1, int c1, const bf16* g, int gc, int li, int P,
                 const Lvl& L, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    FV_CUDA(cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WK * (MAX_CIN + 8 + 64 + 8) * 2));
-    attr = true;
-  }
   WGradArgs a{};
-  a.s0 = s0, a.c0 = c0, a.s1 = s1, a.c1 = c1, a.cin = c0 + c1, a.g = g, a.gc = gc;
+  a.s0 = s0, a.c0 = c0, a.s1 = s1, a.c1 = c1, a.g = g;
   a.ci = n->L[li].ci, a.co = n->L[li].co, a.part = n->wpart;
   a.P = P, a.L = L;
-  if ((a.cin / 16) * (gc / 16) > 4 * WG_PAIRS) return set_error("fv_net: weight-gradient tile too large"), FV_EINVAL;
+  a.pw = std::min(L.X, WK) + 2;
+  a.nr = WK % L.X == 0 ? WK / L.X : (WK - 1) / L.X + 2;
   const long long V = L.cells(P), nchunk = (V + WK - 1) / WK;
   const long long groups = std::min<long long>(nchunk, WG_GROUPS);
   a.chunks_per_cta = (nchunk + groups - 1) / groups;
   const int ng = (int)((nchunk + a.chunks_per_cta - 1) / a.chunks_per_cta);
-  wgrad_kernel<<<dim3(ng, 27), CONV_THREADS, (size_t)WK * (a.cin + 8 + gc + 8) * 2, st>>>(a);
-  wsum_kernel<<<gridsz(27LL * a.ci * a.co, 256), 256, 0, st>>>(n->wpart, ng, a.ci, a.co, n->g + n->L[li].woff);
+  fv_status rc;
+  const int cin = c0 + c1;
+  if (cin == 16 && gc == 16) rc = wgrad_launch<16, 16>(a, cin, ng, st);
+  else if (cin == 16 && gc == 32) rc = wgrad_launch<16, 32>(a, cin, ng, st);
+  else if (cin % 32 == 0 && gc == 16) rc = wgrad_launch<32, 16>(a, cin, ng, st);
+  else if (cin % 32 == 0 && gc == 32) rc = wgrad_launch<32, 32>(a, cin, ng, st);
+  else return set_error("fv_net: unsupported weight-gradient shape"), FV_EINVAL;
+  if (rc) return rc;
+  wsum_kernel<<<gridsz(27LL * a.ci * a.co, 64), 64, 0, st>>>(n->wpart, ng, a.ci, a.co, n->g + n->L[li].woff);
   const int rows = RED_THREADS / gc, nbk = std::min(gridsz(V, rows) / 4 + 1, BG_BLOCKS);
   bgrad_kernel<<<nbk, RED_THREADS, 0, st>>>(g, gc, a.co, P, L, n->bpart);
   bsum_kernel<<<1, 64, 0, st>>>(n->bpart, nbk, a.co, n->g + n->L[li].boff);
@@ -827,8 +983,8 @@ void halo_adj(fv_net* n, bf16* g, int C, int P, const Lvl& L, cudaStream_t st) {
   halo_adjoint_kernel<<<gridsz((long long)P * L.Z * ne * C, 256), 256, 0, st>>>(g, C, P, L, n->halo);
 }
 
-void mask(bf16* g, const bf16* a, int C, int P, const Lvl& L, cudaStream_t st) {
-  mask_kernel<<<gridsz(L.vox(P) * C, 256), 256, 0, st>>>(g, a, C, P, L);
+void mask(const bf16* g, const bf16* a, bf16* out, int C, int P, const Lvl& L, cudaStream_t st) {
+  mask_kernel<<<gridsz(L.vox(P) * (C / 8), 256), 256, 0, st>>>(g, a, out, C, P, L);
 }
 
 fv_status check_nb(const fv_net* n, int nb) {
@@ -911,17 +1067,16 @@ fv_status loss_grad_dev(fv_net* n, int nb, const double* r, const double* e, cud
   const Lvl& L0 = n->lv[0];
   FV_CUDA(cudaMemsetAsync(n->loss, 0, sizeof(double), st));
   FV_CUDA(cudaMemsetAsync(n->g, 0, n->nparam * sizeof(float), st));
-  loss_kernel<<<gridsz(n->V1 * nb, RED_THREADS) / 4 + 1, RED_THREADS, 0, st>>>(
-      n->y, e, n->ss, n->V1, nb, L0, 1.0 / (2.0 * (double)(n->V1 * nb)), n->gy, n->loss);
+  loss_kernel<<<dim3(std::min(gridsz(n->V1, RED_THREADS) / 4 + 1, 2432 / nb + 1), nb), RED_THREADS, 0, st>>>(
+      n->y, e, n->ss, n->V1, L0, 1.0 / (2.0 * (double)(n->V1 * nb)), n->gy, n->loss);
   // output convolution: gradient of its input, D_0 (or E_0 without levels)
   const bf16* last = Lv > 0 ? n->D[0] : n->E[0];
   if ((rc = conv(bwd_args(n->gy, n->L[outL(n)], n->T, P, L0), st)) ||
       (rc = wgrad(n, last, C, nullptr, 0, n->gy, 16, outL(n), P, L0, st)))
     return rc;
   halo_adj(n, n->T, C, P, L0, st);
-  FV_CUDA(cudaMemcpyAsync(Lv > 0 ? n->gD[0] : n->gE[0], n->T, L0.vox(P) * C * sizeof(bf16), cudaMemcpyDeviceToDevice,
-                          st));
-  if (Lv > 0) mask(n->gD[0], n->D[0], C, P, L0, st);
+  if (Lv > 0) mask(n->T, n->D[0], n->gD[0], C, P, L0, st);
+  else FV_CUDA(cudaMemcpyAsync(n->gE[0], n->T, L0.vox(P) * C * sizeof(bf16), cudaMemcpyDeviceToDevice, st));
   // decoder, in reverse order of the forward pass
   for (int l = 0; l < Lv; ++l) {
     const Lvl& L = n->lv[l];
@@ -932,26 +1087,25 @@ fv_status loss_grad_dev(fv_net* n, int nb, const double* r, const double* e, cud
     halo_adj(n, n->T, 2 * C, P, L, st);
     bf16* gnext = l + 1 == Lv ? n->gE[Lv] : n->gD[l + 1];
     const bf16* mk = l + 1 == Lv ? nullptr : n->D[l + 1];
-    split_kernel<<<gridsz(n->lv[l + 1].cells(P) * C, 256), 256, 0, st>>>(n->T, n->gE[l], gnext, mk, C, P, n->lv[l + 1]);
+    split_kernel<<<gridsz(n->lv[l + 1].cells(P) * (C / 8), 256), 256, 0, st>>>(n->T, n->gE[l], gnext, mk, C, P, n->lv[l + 1]);
   }
   // encoder, from the bottom level up
   for (int l = Lv; l >= 0; --l) {
     const Lvl& L = n->lv[l];
-    mask(n->gE[l], n->E[l], C, P, L, st);
+    mask(n->gE[l], n->E[l], n->gE[l], C, P, L, st);
     if ((rc = conv(bwd_args(n->gE[l], n->L[eB(l)], n->T, P, L), st)) ||
         (rc = wgrad(n, n->A[l], C, nullptr, 0, n->gE[l], C, eB(l), P, L, st)))
       return rc;
     halo_adj(n, n->T, C, P, L, st);
     bf16* gA = n->gD[l];  // free at this point: holds the gradient of A_l's pre-activation
-    FV_CUDA(cudaMemcpyAsync(gA, n->T, L.vox(P) * C * sizeof(bf16), cudaMemcpyDeviceToDevice, st));
-    mask(gA, n->A[l], C, P, L, st);
+    mask(n->T, n->A[l], gA, C, P, L, st);
     const bf16* in = l > 0 ? n->In[l] : n->x0;
     const int cin = l > 0 ? C : 16;
     if ((rc = wgrad(n, in, cin, nullptr, 0, gA, C, eA(l), P, L, st))) return rc;
     if (l > 0) {
       if ((rc = conv(bwd_args(gA, n->L[eA(l)], n->T, P, L), st))) return rc;
       halo_adj(n, n->T, C, P, L, st);
-      unpool_add_kernel<<<gridsz(n->lv[l - 1].cells(P) * C, 256), 256, 0, st>>>(n->T, n->gE[l - 1], C, P, L);
+      unpool_add_kernel<<<gridsz(n->lv[l - 1].cells(P) * (C / 8), 256), 256, 0, st>>>(n->T, n->gE[l - 1], C, P, L);
     }
   }
   FV_CUDA(cudaGetLastError());
