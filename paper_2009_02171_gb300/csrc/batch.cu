@@ -66,85 +66,6 @@ void free_batch(BatchWork* b) {
   delete b;
 }
 
-// ------------------------------------------------------------------ batched operator
-template <class GT>
-__global__ void ghost_batch_kernel(GT G, const double* __restrict__ x, double* __restrict__ gh, int d, long long xs,
-                                   long long gsz) {
-  const int Ns = G.Ns, Nr = G.Nr;
-  x += blockIdx.y * xs;
-  gh += blockIdx.y * gsz;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < gsz; e += (long long)gridDim.x * blockDim.x) {
-    long long q = e;
-    const int tp = (int)(q % (Ns + 2));
-    q /= (Ns + 2);
-    const int k = (int)(q % Nr);
-    q /= Nr;
-    const int side = (int)(q % 4);
-    q /= 4;
-    const int p = (int)(q % 6);
-    const int comp = (int)(q / 6);
-    const int t = tp - 1;
-    double v = 0.0;
-    if (t >= 0 && t < Ns) {
-      v = interp_ghost(G, x, comp, p, side, k, t);
-    } else if (side == XI_MIN || side == XI_MAX) {
-      const int jin = t < 0 ? 0 : Ns - 1, iin = side == XI_MIN ? 0 : Ns - 1;
-      v = interp_ghost(G, x, comp, p, side, k, jin) + interp_ghost(G, x, comp, p, t < 0 ? ETA_MIN : ETA_MAX, k, iin) -
-          x[comp * G.N + cidx(G, p, k, jin, iin)];
-    }
-    gh[e] = v;
-  }
-}
-
-// grid.z = ((rhs * d) + comp) * 6 + panel
-template <int KIND, bool INTERIOR>
-__global__ void __launch_bounds__(256) apply_batch_kernel(Geo G, Coefs<double> cf, const double* __restrict__ x,
-                                                          const double* __restrict__ gh, double* __restrict__ y, int d,
-                                                          long long xs, long long ys, long long gsz) {
-  const int Ns = G.Ns;
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  int i, j;
-  if (INTERIOR) {
-    const int ni = Ns - 2;
-    if (q >= ni * ni) return;
-    i = 1 + q % ni, j = 1 + q / ni;
-  } else {
-    if (q >= 4 * (Ns - 1)) return;
-    const int s = q / (Ns - 1), t = q % (Ns - 1);
-    if (s == 0) i = t, j = 0;
-    else if (s == 1) i = Ns - 1, j = t;
-    else if (s == 2) i = Ns - 1 - t, j = Ns - 1;
-    else i = 0, j = Ns - 1 - t;
-  }
-  const int k = blockIdx.y, p = blockIdx.z % 6, ta = blockIdx.z / 6, a = ta % d, rhs = ta / d;
-  ApplyAcc<double, double> acc(G, x + rhs * xs, gh + rhs * gsz);
-  if (KIND == FV_VTBE) vtbe_row(G, cf, acc, p, k, j, i, a);
-  else ppbe_row(G, cf, acc, p, k, j, i, a);
-  y[rhs * ys + (long long)a * G.N + ((long long)(p * G.Nr + k) * Ns + j) * Ns + i] = acc.sum;
-}
-
-static fv_status apply_batch(const fv_system* s, BatchWork* bw, int nrhs, const double* x, long long xs, double* y,
-                             long long ys, cudaStream_t st) {
-  const Geo& G = s->grid->geo;
-  const long long gsz = (long long)s->d * 6 * 4 * G.Nr * (G.Ns + 2);
-  ProfScope ps((s->kind == FV_VTBE ? FV_K_APPLY_VTBE : FV_K_APPLY_PPBE), st);
-  ghost_batch_kernel<Geo><<<dim3((unsigned)std::min<long long>((gsz + 255) / 256, 4096), nrhs), 256, 0, st>>>(
-      G, x, bw->gh, s->d, xs, gsz);
-  const Coefs<double> cf = make_coefs<double>(Phys{s->phys.E, s->phys.Ra, s->phys.Pr, s->phys.Pm, s->phys.dt},
-                                               s->grid->h.ri, s->grid->h.ro);
-  const int ni = G.Ns - 2;
-  const dim3 gi((ni * ni + 255) / 256, G.Nr, 6 * s->d * nrhs), ge((4 * (G.Ns - 1) + 255) / 256, G.Nr, 6 * s->d * nrhs);
-  if (s->kind == FV_VTBE) {
-    apply_batch_kernel<FV_VTBE, true><<<gi, 256, 0, st>>>(G, cf, x, bw->gh, y, s->d, xs, ys, gsz);
-    apply_batch_kernel<FV_VTBE, false><<<ge, 256, 0, st>>>(G, cf, x, bw->gh, y, s->d, xs, ys, gsz);
-  } else {
-    apply_batch_kernel<FV_PPBE, true><<<gi, 256, 0, st>>>(G, cf, x, bw->gh, y, s->d, xs, ys, gsz);
-    apply_batch_kernel<FV_PPBE, false><<<ge, 256, 0, st>>>(G, cf, x, bw->gh, y, s->d, xs, ys, gsz);
-  }
-  FV_CUDA(cudaGetLastError());
-  return FV_OK;
-}
-
 // ------------------------------------------------------------------ batched RAS
 __device__ __forceinline__ void tables(int nx, int ny, int nz, int levels, int* lvl, int* rowoff) {
   for (int L = threadIdx.x; L < levels; L += blockDim.x) {
@@ -650,7 +571,7 @@ static fv_status batch_residual(const fv_system* s, BatchWork* bw, int nrhs, con
   const long long n = s->n;
   const dim3 gv(bblocks(n), nrhs), gc(BBLOCKS, nrhs);
   fv_status rc;
-  if ((rc = apply_batch(s, bw, nrhs, X, n, bw->r, n, st))) return rc;
+  if ((rc = apply_op_batch(s, nrhs, X, n, bw->r, n, bw->gh, st))) return rc;
   scale_batch_kernel<<<gv, 256, 0, st>>>(n, nullptr, bw->r, n, 1.0, B, bw->r, n);
   cgs_batch_dispatch(0, gc, n, bw->r, n, bw->h, bw->r, bw->part, bw->h, bw->ticket, 2, st,
                      std::make_integer_sequence<int, BK>{});
@@ -675,7 +596,7 @@ static fv_status batch_cycle(const fv_system* s, BatchWork* bw, int nrhs, const 
     double* zj = bw->Z + (size_t)j * n;
     // Z_j = M^{-1} V_j and w = A Z_j for every right-hand side (strided in the bases)
     if ((rc = ras_batch(s, bw, nrhs, vj, vs, zj, zs, st))) return rc;
-    if ((rc = apply_batch(s, bw, nrhs, zj, zs, bw->w, n, st))) return rc;
+    if ((rc = apply_op_batch(s, nrhs, zj, zs, bw->w, n, bw->gh, st))) return rc;
     const int nv = j + 1;
     {
       ProfScope ps(FV_K_CGS, st);

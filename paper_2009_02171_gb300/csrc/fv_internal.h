@@ -225,8 +225,11 @@ fv_status build_grid(const fv_grid_desc* desc, fv_grid** out);
 void free_grid(fv_grid* g);
 
 // apply.cu (tiled operator apply), ops.cu
-fv_status apply_op(const fv_system* s, const double* x, double* y, cudaStream_t st);
-fv_status apply_op32(const fv_system* s, const float* x, float* y, cudaStream_t st);
+// y = A x, or y = b - A x when b is given
+fv_status apply_op(const fv_system* s, const double* x, double* y, cudaStream_t st, const double* b = nullptr);
+fv_status apply_op32(const fv_system* s, const float* x, float* y, cudaStream_t st, const float* b = nullptr);
+fv_status apply_op_batch(const fv_system* s, int nrhs, const double* x, long long xs, double* y, long long ys, double* E,
+                         cudaStream_t st);
 fv_status apply_op_noalloc(const fv_system* s, const double* x, double* y, cudaStream_t st);
 fv_status ghost_fill(const Geo& G, const double* x, double* gh, int d, cudaStream_t st);
 fv_status assemble_subdomains(fv_system* s);

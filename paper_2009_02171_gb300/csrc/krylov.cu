@@ -911,14 +911,6 @@ fv_status to_fp64(long long n, const float* x, double* out, cudaStream_t st) {
   return FV_OK;
 }
 
-template <class T>
-static fv_status axpby_t(long long n, double a, const T* x, double b, const T* y, T* out, cudaStream_t st) {
-  ProfScope ps(FV_K_VEC, st);
-  axpby_kernel<T, T><<<vblocks(n), 256, 0, st>>>(n, a, x, b, y, out);
-  FV_CUDA(cudaGetLastError());
-  return FV_OK;
-}
-
 // ||x||, and x / ||x|| into vout (null: none)
 template <class T>
 static fv_status norm2(KrylovT<T>& k, long long n, const T* x, T* vout, cudaStream_t st, double* out) {
@@ -929,15 +921,16 @@ static fv_status norm2(KrylovT<T>& k, long long n, const T* x, T* vout, cudaStre
   return FV_OK;
 }
 
+// y = A x, or y = b - A x
 template <class T>
-static fv_status apply_t(const fv_system* s, const T* x, T* y, cudaStream_t st);
+static fv_status apply_t(const fv_system* s, const T* x, T* y, cudaStream_t st, const T* b = nullptr);
 template <>
-fv_status apply_t<double>(const fv_system* s, const double* x, double* y, cudaStream_t st) {
-  return apply_op(s, x, y, st);
+fv_status apply_t<double>(const fv_system* s, const double* x, double* y, cudaStream_t st, const double* b) {
+  return apply_op(s, x, y, st, b);
 }
 template <>
-fv_status apply_t<float>(const fv_system* s, const float* x, float* y, cudaStream_t st) {
-  return apply_op32(s, x, y, st);
+fv_status apply_t<float>(const fv_system* s, const float* x, float* y, cudaStream_t st, const float* b) {
+  return apply_op32(s, x, y, st, b);
 }
 
 template <class T>
@@ -1028,8 +1021,7 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
   const int lvl = FV_K_COARSE * s->level + (sizeof(T) == 4 ? FV_K_FP32 : 0);
   if (!inner) s->last_inner = 0;
   // r = b - A x
-  if ((rc = apply_t<T>(s, x, k.r, st))) return rc;
-  if ((rc = axpby_t<T>(n, 1.0, b, -1.0, k.r, k.r, st))) return rc;
+  if ((rc = apply_t<T>(s, x, k.r, st, b))) return rc;
   double beta;
   if ((rc = norm2<T>(k, n, k.r, k.V, st, &beta))) return rc;
   const double r0 = beta, target = std::max(o->atol, o->rtol * r0);
@@ -1095,8 +1087,7 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
       update_dispatch<T>(kk, vblocks(n), n, k.Z, c, x, st, std::make_integer_sequence<int, KMAX>{});
       FV_CUDA(cudaGetLastError());
     }
-    if ((rc = apply_t<T>(s, x, k.r, st))) return rc;
-    if ((rc = axpby_t<T>(n, 1.0, b, -1.0, k.r, k.r, st))) return rc;
+    if ((rc = apply_t<T>(s, x, k.r, st, b))) return rc;
     if ((rc = norm2<T>(k, n, k.r, k.V, st, &beta))) return rc;
     if (!std::isfinite(beta)) nan = true;
     if (breakdown) break;

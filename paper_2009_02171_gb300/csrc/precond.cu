@@ -875,8 +875,7 @@ fv_status precond_apply(const fv_system* s, const double* r, double* z, cudaStre
     ProfScope ph(FV_K_PHASE_PC_I, st);
     if ((rc = prolong_inject(s->grid, s->d, s->ec, s->w, st))) return rc;
     // y = w + M_one^{-1} (r - A_f w)   (eqn:finesolve)
-    if ((rc = apply_op(s, s->w, s->t, st))) return rc;
-    if ((rc = axpby(s->n, 1.0, r, -1.0, s->t, s->t, st))) return rc;
+    if ((rc = apply_op(s, s->w, s->t, st, r))) return rc;
   }
   {
     ProfScope ph(FV_K_PHASE_PC_F, st);
@@ -903,7 +902,7 @@ fv_status precond_apply32(const fv_system* s, const float* r, float* z, cudaStre
       // learned e_c = N(r_c), then learned_its iterations on the residual r_c - A_c e_c
       if ((rc = net_forward32(s->net, s->xc32, s->ec32, st))) return rc;
       if (s->learned_its > 0) {
-        if ((rc = apply_op32(c, s->ec32, s->tc32, st)) || (rc = axpby32(c->n, 1.0, s->xc32, -1.0, s->tc32, s->tc32, st)) ||
+        if ((rc = apply_op32(c, s->ec32, s->tc32, st, s->xc32)) ||
             (rc = gmres_fixed32(c, s->tc32, s->dc32, s->learned_its, st)) ||
             (rc = axpby32(c->n, 1.0, s->ec32, 1.0, s->dc32, s->ec32, st)))
           return rc;
@@ -915,8 +914,7 @@ fv_status precond_apply32(const fv_system* s, const float* r, float* z, cudaStre
   {
     ProfScope ph(FV_K_PHASE_PC_I, st);
     if ((rc = prolong_t<float>(s->grid, s->d, s->ec32, s->w32, st))) return rc;
-    if ((rc = apply_op32(s, s->w32, s->t32, st))) return rc;
-    if ((rc = axpby32(s->n, 1.0, r, -1.0, s->t32, s->t32, st))) return rc;
+    if ((rc = apply_op32(s, s->w32, s->t32, st, r))) return rc;
   }
   {
     ProfScope ph(FV_K_PHASE_PC_F, st);
@@ -948,7 +946,7 @@ void set_learned_active(fv_system* s, int on) {
 // x <- x + I_c^f N(r_c(b - A x)): the learned initial-guess correction
 fv_status learned_guess(const fv_system* s, const double* b, double* x, cudaStream_t st) {
   fv_status rc;
-  if ((rc = apply_op(s, x, s->t, st)) || (rc = axpby(s->n, 1.0, b, -1.0, s->t, s->t, st)) ||
+  if ((rc = apply_op(s, x, s->t, st, b)) ||
       (rc = restrict_coarse(s, s->t, s->xc, st)) || (rc = net_forward64(s->net, s->xc, s->ec, st)) ||
       (rc = prolong_inject(s->grid, s->d, s->ec, s->w, st)))
     return rc;
