@@ -25,7 +25,10 @@
 namespace fv {
 
 constexpr int BK = 32;        // max basis vectors
-constexpr int BBLOCKS = 152;  // reduction blocks per right-hand side
+constexpr int BBLOCKS = 152;  // reduction blocks per right-hand side at most
+// about four blocks an SM over all right-hand sides: every block adds a reduction of its FP64 partial sums (five
+// DADDs a warp and value on the slow pipe), which with 152 blocks a right-hand side was over half of a pass
+static int rblocks(int nrhs) { return std::max(16, std::min(BBLOCKS, 608 / nrhs)); }
 constexpr int BTHREADS = 256;
 
 // device-side Arnoldi bookkeeping of one right-hand side (Hessenberg column-major H[j * BK + i])
@@ -374,18 +377,26 @@ __global__ void __launch_bounds__(BTHREADS) cgs_batch_kernel(long long n, const 
       nrm += we * we;
     }
   }
-  __shared__ double sm[BTHREADS / 32][BK];
+  // eight values at a time through shared memory: a warp adds eight partial sums a lane, then its butterfly
+  __shared__ double red[8][BTHREADS];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nvv = mode < 2 ? NV : 1;
-  for (int v = 0; v < nvv; ++v) {
-    const double t = bwarp_sum(mode < 2 ? acc[v] : nrm);
-    if (lane == 0) sm[wid][v] = t;
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < nvv) {
-    double t = 0.0;
-    for (int q = 0; q < BTHREADS / 32; ++q) t += sm[q][threadIdx.x];
-    part[threadIdx.x * gridDim.x + blockIdx.x] = t;
+  if (mode == 2) acc[0] = nrm;
+#pragma unroll
+  for (int v0 = 0; v0 < (NV > 0 ? NV : 1); v0 += 8) {
+    if (v0 >= nvv) break;
+    if (v0) __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (v0 + u < (NV > 0 ? NV : 1)) red[u][threadIdx.x] = acc[v0 + u < (NV > 0 ? NV : 1) ? v0 + u : 0];
+    __syncthreads();
+    if (v0 + wid < nvv) {
+      double t = 0.0;
+#pragma unroll
+      for (int u = 0; u < BTHREADS / 32; ++u) t += red[wid][32 * u + lane];
+      t = bwarp_sum(t);
+      if (lane == 0) part[(v0 + wid) * gridDim.x + blockIdx.x] = t;
+    }
   }
   __shared__ bool last;
   __threadfence();
@@ -569,7 +580,7 @@ __global__ void batch_lsq_kernel(int nrhs, BatchArn* __restrict__ arn, double* _
 static fv_status batch_residual(const fv_system* s, BatchWork* bw, int nrhs, const double* B, const double* X,
                                 const fv_gmres_opts* o, int first, cudaStream_t st) {
   const long long n = s->n;
-  const dim3 gv(bblocks(n), nrhs), gc(BBLOCKS, nrhs);
+  const dim3 gv(bblocks(n), nrhs), gc(rblocks(nrhs), nrhs);
   fv_status rc;
   if ((rc = apply_op_batch(s, nrhs, X, n, bw->r, n, bw->gh, st))) return rc;
   scale_batch_kernel<<<gv, 256, 0, st>>>(n, nullptr, bw->r, n, 1.0, B, bw->r, n);
@@ -588,7 +599,7 @@ static fv_status batch_cycle(const fv_system* s, BatchWork* bw, int nrhs, const 
   const int m = o->restart;
   const long long n = s->n;
   const long long vs = (long long)(m + 1) * n, zs = (long long)m * n;
-  const dim3 gv(bblocks(n), nrhs), gc(BBLOCKS, nrhs);
+  const dim3 gv(bblocks(n), nrhs), gc(rblocks(nrhs), nrhs);
   fv_status rc;
   scale_batch_kernel<<<gv, 256, 0, st>>>(n, bw->coef, bw->r, n, 0.0, nullptr, bw->V, vs);
   for (int j = 0; j < m; ++j) {
