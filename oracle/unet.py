@@ -220,10 +220,13 @@ def loss_and_grads(params, r, e, levels):
     L = float((diff * diff).mean())
     gy = 2.0 * diff / diff.size
     grads = {}
-    gxp, gw, gb = conv_backward(pad(c['D'][0]), params['out'][0], gy)
+    last = c['D'][0] if levels else c['E'][0]  # without a coarser level the output layer reads the encoder
+    gxp, gw, gb = conv_backward(pad(last), params['out'][0], gy)
     grads['out'] = (gw, gb)
-    gd = pad_adjoint(gxp) * (c['D'][0] > 0)
+    gd = pad_adjoint(gxp) * (last > 0)
     gE = [np.zeros_like(E) for E in c['E']]
+    if not levels:
+        gE[0] += gd
     C = c['E'][0].shape[1]
     # decoder in reverse order of the forward pass: l = 0 .. levels-1
     cats = {l: c['cat'][levels - 1 - l] for l in range(levels)}
