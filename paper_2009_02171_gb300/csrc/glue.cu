@@ -121,44 +121,89 @@ __device__ __noinline__ void edge_face_flux(const Geo& G, const Field& F, double
   for (int m = 0; m < NO; ++m) out[m] = 0.5 * (a[m] + sg * b[m]);
 }
 
+// components of the field a mode reads
+template <int MODE>
+__host__ __device__ constexpr int field_comp(int m) { return MODE == MODE_DIV && m >= 3 ? m + 1 : m; }
+template <int MODE>
+__host__ __device__ constexpr int field_count() { return MODE == MODE_NL ? 7 : MODE == MODE_DIV ? 6 : 2; }
+
+// acc += a (flux through a face), from twice the face means w2 (the values of both cells added) and the tabulated face
+// vector l: the factor of the means (1/2 or 1/4) and, for the four horizontal faces, r_k stay with the cell's scale.
+template <int MODE, int NO>
+__device__ __forceinline__ void add_flux(double a, double cL, const double* w2, const double* __restrict__ l, double (&acc)[NO]) {
+  const double S0 = l[0], S1 = l[1], S2 = l[2];
+  if constexpr (MODE == MODE_NL) {
+    const double un = -a * (w2[0] * S0 + w2[1] * S1 + w2[2] * S2);
+    const double bn = a * (w2[4] * S0 + w2[5] * S1 + w2[6] * S2), bc = cL * bn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      acc[c] = fma(un, w2[c], acc[c]), acc[c] = fma(bc, w2[4 + c], acc[c]);
+      acc[4 + c] = fma(bn, w2[c], acc[4 + c]), acc[4 + c] = fma(un, w2[4 + c], acc[4 + c]);
+    }
+    acc[3] = fma(un, w2[3], acc[3]);
+  } else if constexpr (MODE == MODE_DIV) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) acc[q] = fma(a, w2[3 * q] * S0 + w2[3 * q + 1] * S1 + w2[3 * q + 2] * S2, acc[q]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double t = a * w2[q];
+      acc[3 * q] = fma(t, S0, acc[3 * q]), acc[3 * q + 1] = fma(t, S1, acc[3 * q + 1]), acc[3 * q + 2] = fma(t, S2, acc[3 * q + 2]);
+    }
+  }
+}
+
 // Interior and radial faces of every cell (panel-edge faces contribute zero here and are added by
 // edge_face_kernel, so no warp of this kernel waits on the ghost interpolation of an edge cell).
+// Bound by the FP64 pipe (16 cycles of an SM a warp instruction), not by its bytes: sums instead of means, the
+// common factors taken out of the face and products accumulated directly leave 28 operations a face of the nonlinear
+// terms, against 53 when every face's flux was formed and then added.  Mean of the
+// nonlinear, divergence and gradient launches, edge faces included: 6x64^3 509 -> 361 us, 6x128^2x96 3.02 -> 2.05 ms
 // grid: x = tiles of the (j, i) plane, y = k, z = panel
 template <int MODE, int NO>
-__global__ void face_kernel(Geo G, Field F, double cL, double scale, double* __restrict__ out) {
+__global__ void __launch_bounds__(128) face_kernel(Geo G, Field F, double cL, double scale, double* __restrict__ out) {
+  constexpr int NF = field_count<MODE>();
   const int Ns = G.Ns;
   const int ij = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ij < Ns * Ns) {
-    const int i = ij % Ns, j = ij / Ns, k = blockIdx.y, p = blockIdx.z;
-    const long long e = ((long long)(p * G.Nr + k) * Ns + j) * Ns + i;
-    double acc[NO], fl[7];
-    for (int m = 0; m < NO; ++m) acc[m] = 0.0;
-    // xi faces
-    if (i + 1 < Ns) {
-      face_flux<MODE>(G, F, cL, p, 0, k, j, i + 1, fl);
-      for (int m = 0; m < NO; ++m) acc[m] += fl[m];
+  if (ij >= Ns * Ns) return;
+  const int i = ij % Ns, j = ij / Ns, k = blockIdx.y, p = blockIdx.z;
+  const long long e = ((long long)(p * G.Nr + k) * Ns + j) * Ns + i;
+  double acc[NO], xc[NF], w2[7];
+#pragma unroll
+  for (int m = 0; m < NO; ++m) acc[m] = 0.0;
+#pragma unroll
+  for (int m = 0; m < NF; ++m) xc[m] = F.x[field_comp<MODE>(m) * G.N + e];
+  // the face towards the cell at distance d of the same panel
+  auto face = [&](long long d, const double* l, double a) {
+#pragma unroll
+    for (int m = 0; m < NF; ++m) w2[m] = xc[m] + F.x[field_comp<MODE>(m) * G.N + e + d];
+    add_flux<MODE, NO>(a, cL, w2, l, acc);
+  };
+  const double* lx = G.sxp + 3 * (((long long)p * Ns + j) * (Ns + 1) + i);
+  const double* ly = G.syp + 3 * (((long long)p * (Ns + 1) + j) * Ns + i);
+  if (i + 1 < Ns) face(1, lx + 3, 1.0);
+  if (i > 0) face(-1, lx, -1.0);
+  if (j + 1 < Ns) face(Ns, ly + 3 * Ns, 1.0);
+  if (j > 0) face(-Ns, ly, -1.0);
+  const double rk = G.rc[k];
+#pragma unroll
+  for (int m = 0; m < NO; ++m) acc[m] *= rk;
+  const double* lr = G.srp + 3 * (((long long)p * Ns + j) * Ns + i);
+  const long long up = (long long)Ns * Ns;
+#pragma unroll
+  for (int side = 1; side >= 0; --side) {
+    const double a = side ? G.rf2[k + 1] : -G.rf2[k];
+    if (side ? k + 1 < G.Nr : k > 0) {
+      face(side ? up : -up, lr, a);
+    } else {
+#pragma unroll
+      for (int m = 0; m < NF; ++m) w2[m] = 2.0 * face_val_any(G, F, field_comp<MODE>(m), p, 2, k + side, j, i);
+      add_flux<MODE, NO>(a, cL, w2, lr, acc);
     }
-    if (i > 0) {
-      face_flux<MODE>(G, F, cL, p, 0, k, j, i, fl);
-      for (int m = 0; m < NO; ++m) acc[m] -= fl[m];
-    }
-    // eta faces
-    if (j + 1 < Ns) {
-      face_flux<MODE>(G, F, cL, p, 1, k, j + 1, i, fl);
-      for (int m = 0; m < NO; ++m) acc[m] += fl[m];
-    }
-    if (j > 0) {
-      face_flux<MODE>(G, F, cL, p, 1, k, j, i, fl);
-      for (int m = 0; m < NO; ++m) acc[m] -= fl[m];
-    }
-    // radial faces
-    face_flux<MODE>(G, F, cL, p, 2, k + 1, j, i, fl);
-    for (int m = 0; m < NO; ++m) acc[m] += fl[m];
-    face_flux<MODE>(G, F, cL, p, 2, k, j, i, fl);
-    for (int m = 0; m < NO; ++m) acc[m] -= fl[m];
-    const double iv = scale * G.invsig[j * Ns + i] * G.invr2[k];
-    for (int m = 0; m < NO; ++m) out[m * G.N + e] = acc[m] * iv;
   }
+  const double iv = (MODE == MODE_NL ? 0.25 : 0.5) * scale * G.invsig[j * Ns + i] * G.invr2[k];
+#pragma unroll
+  for (int m = 0; m < NO; ++m) out[m * G.N + e] = acc[m] * iv;
 }
 
 // Panel-edge faces (the mean of the two panels' one-sided fluxes), added to the cells that own
