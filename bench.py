@@ -66,8 +66,7 @@ METRIC = 'wall time per time step at 1e-8 residual'
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a kernel category at the default
 # workload, from the ncu capture in the file named beside it; a category leaves this table when its kernels
 # change, until they are captured again
-TRAFFIC = {'net_fwd': (49537707, 'profiles/launches_net_forward_c16_coarse32.md'),
-           'apply_vtbe_fp32': (57991936, 'profiles/ncu_apply_vtbe_fp32_shell64.md')}
+TRAFFIC = {}
 # CPU oracle: wall-clock budget for its real time steps (after its setup); at least one step always runs
 ORACLE_BUDGET_S = float(os.environ.get('FV_ORACLE_BUDGET_S', '100'))
 
@@ -347,8 +346,8 @@ def net_workload(args, fv, torch, rank, ws):
                           'gpu_launches': args.steps * (8 + 5 * L['levels']),
                           'roofline': {'kernel': 'net_fwd', 'bound': 'tensor', 'achieved': round(ach, 2), 'peak': pk,
                                        'unit': 'TFLOP/s', 'frac': round(ach / pk, 4),
-                                       'traffic': TRAFFIC['net_fwd'][0] if not args.ns else None,
-                                       'traffic_source': TRAFFIC['net_fwd'][1] if not args.ns else None,
+                                       'traffic': TRAFFIC.get('net_fwd', (None, None))[0] if not args.ns else None,
+                                       'traffic_source': TRAFFIC.get('net_fwd', (None, None))[1] if not args.ns else None,
                                        'flops_per_launch': flops,
                                        'peak_source': 'MEASURED_PEAKS.json bf16_tflops (of measured; timed alone)'}}))
     fv.fv_net_free(net)

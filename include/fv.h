@@ -202,10 +202,12 @@ fv_status fv_gmres_solve(const fv_system* s, const double* b, double* x, const f
  * Hessenberg matrix, tolerance and convergence flag.  B, X: device FP64,
  * nrhs * n values, right-hand side r at offset r * n (X: in = x0, out = x).
  * The preconditioner is the system's one-level RAS (levels = 1 only), with
- * FP32 subdomain solves when the system was assembled with FV_PREC_FP32;
- * every factor the batched sweeps load is applied to a group of right-hand
- * sides (the group size is tuned by timing on the first call for a given
- * nrhs), in one persistent launch that takes subdomains largest first.
+ * FP32 subdomain solves when the system was assembled with FV_PREC_FP32,
+ * one launch over all (subdomain, right-hand side) pairs.  Subdomains too wide
+ * for that (above 384 rows in a wavefront's window): every factor loaded is
+ * applied to a group of right-hand sides (the group size is tuned by timing
+ * on the first call for a given nrhs), in one persistent launch a direction
+ * that takes subdomains largest first.
  * stats: NULL or nrhs entries. */
 fv_status fv_gmres_solve_batch(const fv_system* s, int nrhs, const double* B, double* X, const fv_gmres_opts* opts,
                                fv_solve_stats* stats, void* stream);
@@ -272,7 +274,8 @@ fv_status fv_state_diagnostics(fv_state* st, const fv_system* ppbe, fv_diag* out
  * preconditioner, plus FV_K_FP32 for FP32 launches of mixed precision.  The
  * phases PC-C (coarse solve), PC-F (fine one-level RAS) and PC-I
  * (restriction, prolongation and residual) follow the paper's breakdown of
- * the two-level preconditioner (Sec. 4.3). */
+ * the two-level preconditioner (Sec. 4.3).  Subdomain solves that do both
+ * sweeps in one launch count under the forward category. */
 #define FV_K_GHOST 0
 #define FV_K_APPLY_VTBE 1
 #define FV_K_APPLY_PPBE 2

@@ -8,13 +8,10 @@
 // one-level RAS: FP64 subdomain solves, or FP32 subdomain solves inside the
 // FP64 outer FGMRES when the system was assembled with FV_PREC_FP32.
 //
-// Batched RAS sweeps: each CTA takes a (subdomain, group of G right-hand
-// sides) task and applies every factor it loads to the G right-hand sides,
-// so the factor bytes are read once per group instead of once per
-// right-hand side.  The launch is persistent: as many CTAs as fit on the GPU
-// pull tasks from an atomic counter in decreasing subdomain size (uneven
-// decompositions balance).  G is chosen by timing each candidate on the first
-// call for a given nrhs (an autotuner; the choice is kept in the system).
+// Batched RAS sweeps: the streamed sweeps over (subdomain, right-hand side) tasks.  Subdomains too wide for them: each
+// CTA takes a (subdomain, group of G right-hand sides) task and applies every factor it loads to the G right-hand
+// sides; the launch is persistent, as many CTAs as fit on the GPU pull tasks from an atomic counter in decreasing
+// subdomain size, and G is chosen by timing each candidate on the first call for a given nrhs (kept in the system).
 #include <algorithm>
 #include <chrono>
 #include <cmath>
