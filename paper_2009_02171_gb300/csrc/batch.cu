@@ -34,6 +34,7 @@ struct BatchArn {
   double cs[BK], sn[BK], g[BK + 1], y[BK];
   double beta, r0, target;
   int its, kk, done;
+  int max_it;  // of this solve: kept here, since a captured cycle is replayed by solves with other limits
 };
 
 struct BatchWork {
@@ -503,17 +504,18 @@ static fv_status ensure_batch(const fv_system* s, int nrhs, int m) {
   return setup_ras(s, bw, tab);
 }
 
-// after r = B - A X and its squared norm (h[2 BK] per right-hand side): beta, the target on the first call,
-// the convergence flag, 1 / beta into coef, g = beta e_1 (one thread per right-hand side)
+// after r = B - A X and its squared norm (h[2 BK] per right-hand side): beta, the target and the iteration limit on
+// the first call (atol, rtol and max_it are read there only: a captured cycle holds those of the solve that captured
+// it), the convergence flag, 1 / beta into coef, g = beta e_1 (one thread per right-hand side)
 __global__ void batch_start_kernel(int nrhs, BatchArn* __restrict__ arn, const double* __restrict__ h,
                                    double* __restrict__ coef, int first, double atol, double rtol, int max_it) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nrhs) return;
   BatchArn& a = arn[t];
   const double beta = sqrt(h[t * 3 * BK + 2 * BK]);
-  if (first) a.r0 = beta, a.target = fmax(atol, rtol * beta), a.its = 0;
+  if (first) a.r0 = beta, a.target = fmax(atol, rtol * beta), a.its = 0, a.max_it = max_it;
   a.beta = beta;
-  a.done = !(isfinite(beta) && beta > a.target && a.its < max_it);
+  a.done = !(isfinite(beta) && beta > a.target && a.its < a.max_it);
   a.kk = 0;
   for (int i = 0; i <= BK; ++i) a.g[i] = 0.0;
   for (int i = 0; i < BK; ++i) a.y[i] = 0.0;
@@ -525,7 +527,7 @@ __global__ void batch_start_kernel(int nrhs, BatchArn* __restrict__ arn, const d
 // h_{j+1,j} = sqrt(||w||^2)), previous rotations, a new rotation, the right-hand side update; the next basis
 // vector's scale 1 / h_{j+1,j} into coef, 0 once converged (its later columns are zero and unused)
 __global__ void batch_givens_kernel(int nrhs, int j, BatchArn* __restrict__ arn, const double* __restrict__ h,
-                                    double* __restrict__ coef, int max_it) {
+                                    double* __restrict__ coef) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nrhs) return;
   BatchArn& a = arn[t];
@@ -551,7 +553,7 @@ __global__ void batch_givens_kernel(int nrhs, int j, BatchArn* __restrict__ arn,
   for (int i = 0; i <= j; ++i) a.H[j * BK + i] = col[i];
   ++a.its;
   a.kk = j + 1;
-  if (fabs(a.g[j + 1]) <= a.target || a.its >= max_it || !(hn > 0.0) || !isfinite(hn)) {
+  if (fabs(a.g[j + 1]) <= a.target || a.its >= a.max_it || !(hn > 0.0) || !isfinite(hn)) {
     a.done = 1;
     coef[t] = 0.0;
   } else {
@@ -614,7 +616,7 @@ static fv_status batch_cycle(const fv_system* s, BatchWork* bw, int nrhs, const 
                          std::make_integer_sequence<int, BK>{});
       cgs_batch_dispatch(nv, gc, n, bw->V, vs, bw->h + BK, bw->w, bw->part, bw->h, bw->ticket, 2, st,
                          std::make_integer_sequence<int, BK>{});
-      batch_givens_kernel<<<(nrhs + 31) / 32, 32, 0, st>>>(nrhs, j, bw->arn, bw->h, bw->coef, o->max_it);
+      batch_givens_kernel<<<(nrhs + 31) / 32, 32, 0, st>>>(nrhs, j, bw->arn, bw->h, bw->coef);
     }
     FV_CUDA(cudaGetLastError());
     if (j + 1 < m) scale_batch_kernel<<<gv, 256, 0, st>>>(n, bw->coef, bw->w, n, 0.0, nullptr, bw->V + (size_t)(j + 1) * n, vs);
