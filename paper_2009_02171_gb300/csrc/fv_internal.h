@@ -183,6 +183,7 @@ struct fv_system {
   float *xc32 = nullptr, *ec32 = nullptr, *w32 = nullptr, *t32 = nullptr;  // FP32 two-level work
   cudaGraphExec_t inner_graph = nullptr;  // captured inner solve (r32 -> x32)
   int inner_warm = 0;
+  unsigned long long inner_buffers = 0;   // fv::inner_buffers() when inner_graph was captured
   // FGMRES workspace for this system (outer) sized lazily
   fv::Krylov* kry = nullptr;
   fv::BatchWork* batch = nullptr;  // fv_gmres_solve_batch workspace
@@ -269,6 +270,7 @@ bool net_matches(const fv_net* n, const fv_grid* coarse);
 fv_status gmres(const fv_system* s, const double* b, double* x, const fv_gmres_opts* o, fv_solve_stats* stats,
                 cudaStream_t st, bool inner);
 void free_krylov(Krylov* k);
+unsigned long long inner_buffers(const fv_system* s);
 void free_batch(BatchWork* b);
 fv_status axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st);
 fv_status axpby32(long long n, double a, const float* x, double b, const float* y, float* out, cudaStream_t st);

@@ -60,7 +60,16 @@ struct KrylovT {
 struct Krylov {
   KrylovT<double> d;
   KrylovT<float> f;
+  unsigned long long moves = 0;  // times the FP32 workspace has been allocated
 };
+
+// Changes when a buffer of the FP32 inner solve of s (its own or a coarser level's) is allocated anew: a coarse system
+// is also a system of its own (fv_coarse_system), whose solves may need more vectors than its place in the hierarchy.
+unsigned long long inner_buffers(const fv_system* s) {
+  unsigned long long n = 0;
+  for (; s; s = s->coarse) n += s->kry ? s->kry->moves : 0;
+  return n;
+}
 
 template <class T>
 static void free_kt(KrylovT<T>& k) {
@@ -93,6 +102,7 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
   KrylovT<T>& k = kt<T>(sm->kry);
   if (k.m >= m && k.n == s->n) return FV_OK;
   free_kt(k);
+  if (sizeof(T) == 4) ++sm->kry->moves;
   k.m = m, k.n = s->n;
   const size_t n = (size_t)s->n;
   if (cudaMalloc(&k.V, (m + 1) * n * sizeof(T)) != cudaSuccess || cudaMalloc(&k.Z, m * n * sizeof(T)) != cudaSuccess ||

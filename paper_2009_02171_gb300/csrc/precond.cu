@@ -828,7 +828,8 @@ fv_status prolong_inject(const fv_grid* g, int d, const double* xc, double* x, c
 // inner_maxit iterations (its two-level preconditioner's coarse solve: exactly
 // coarse_maxit iterations), driven on the device.  The sequence r32 -> x32 has fixed
 // buffers and no host synchronisation: it is captured once into a CUDA graph and
-// replayed (kernel timing, when enabled, runs it eagerly instead).
+// replayed (kernel timing, when enabled, runs it eagerly instead).  A graph whose
+// buffers have been allocated anew since is captured again.
 static fv_status inner_sequence(const fv_system* s, cudaStream_t st) {
   return gmres_fixed32(s, s->r32, s->x32, s->pc.inner_maxit, st);
 }
@@ -840,6 +841,10 @@ static fv_status inner_solve(const fv_system* s, const double* r, double* z, cud
     if ((rc = inner_sequence(s, st))) return rc;
   } else {
     fv_system* sm = const_cast<fv_system*>(s);
+    if (sm->inner_graph && sm->inner_buffers != inner_buffers(s)) {
+      FV_CUDA(cudaGraphExecDestroy(sm->inner_graph));
+      sm->inner_graph = nullptr;
+    }
     if (!sm->inner_warm) {
       // first call: run eagerly so every lazily allocated workspace exists before capture
       if ((rc = inner_sequence(s, st))) return rc;
@@ -857,6 +862,7 @@ static fv_status inner_solve(const fv_system* s, const double* r, double* z, cud
       ce = cudaGraphInstantiate(&sm->inner_graph, graph, 0);
       cudaGraphDestroy(graph);
       FV_CUDA(ce);
+      sm->inner_buffers = inner_buffers(s);
     }
     if (sm->inner_graph) FV_CUDA(cudaGraphLaunch(s->inner_graph, st));
   }
