@@ -189,6 +189,14 @@ fv_status fv_gmres_solve(const fv_system* s, const double* b, double* x, const f
   return gmres(s, b, x, opts, stats, (cudaStream_t)stream, false);
 }
 
+fv_status fv_set_wait_limit(fv_system* s, unsigned tries) {
+  if (!s) return set_error("fv_set_wait_limit: null system"), FV_EINVAL;
+  s->wait_limit = tries;
+  if (s->inner_graph) cudaGraphExecDestroy(s->inner_graph);  // holds the limits it was captured with
+  s->inner_graph = nullptr;
+  return FV_OK;
+}
+
 fv_status fv_coarse_system(const fv_system* s, const fv_system** coarse) {
   if (!s || !coarse) return set_error("fv_coarse_system: null argument"), FV_EINVAL;
   if (!s->coarse) return set_error("fv_coarse_system: the system has one level"), FV_EINVAL;

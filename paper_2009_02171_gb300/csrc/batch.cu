@@ -683,7 +683,7 @@ fv_status gmres_batch(const fv_system* s, int nrhs, const double* B, double* X, 
     }
     if ((rc = fetch_state())) return rc;
   }
-  if (sweep_failed(s)) return set_error("fv_gmres_solve_batch: a wait of the subdomain sweeps ran out"), FV_ECUDA;
+  if ((rc = waits_failed(s, "fv_gmres_solve_batch: ", st))) return rc;
   bool all_conv = true, nan = false;
   for (int t = 0; t < nrhs; ++t) {
     const BatchArn& a = bw->arn_host[t];

@@ -184,6 +184,7 @@ struct fv_system {
   cudaGraphExec_t inner_graph = nullptr;  // captured inner solve (r32 -> x32)
   int inner_warm = 0;
   unsigned long long inner_buffers = 0;   // fv::inner_buffers() when inner_graph was captured
+  unsigned wait_limit = 1u << 24;  // tries after which a wait between blocks gives up
   // FGMRES workspace for this system (outer) sized lazily
   fv::Krylov* kry = nullptr;
   fv::BatchWork* batch = nullptr;  // fv_gmres_solve_batch workspace
@@ -271,6 +272,8 @@ fv_status gmres(const fv_system* s, const double* b, double* x, const fv_gmres_o
                 cudaStream_t st, bool inner);
 void free_krylov(Krylov* k);
 unsigned long long inner_buffers(const fv_system* s);
+// after a synchronisation: FV_ECUDA if a bounded wait of s or of its coarse levels ran out since the last call
+fv_status waits_failed(const fv_system* s, const char* where, cudaStream_t st);
 void free_batch(BatchWork* b);
 fv_status axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st);
 fv_status axpby32(long long n, double a, const float* x, double b, const float* y, float* out, cudaStream_t st);
@@ -283,3 +286,6 @@ fv_status weighted_mean_remove32(const fv_grid* g, float* x, cudaStream_t st, do
 fv_status weighted_mean_remove(const fv_grid* g, double* x, cudaStream_t st, double* part, double* sums);
 
 }  // namespace fv
+
+// For tests of the reporting, not in the public headers: the tries after which a grid barrier of s (this level) gives up.
+extern "C" fv_status fv_set_wait_limit(fv_system* s, unsigned tries);

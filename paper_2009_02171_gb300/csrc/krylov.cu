@@ -52,8 +52,9 @@ struct KrylovT {
   double* hhost = nullptr;  // pinned [3][KMAX]
   ArnoldiDev* ad = nullptr; // device-driven solves
   unsigned* ticket = nullptr; // last-block counter of the fused reductions (returns to 0 after each use)
-  unsigned* bar = nullptr;    // [2] grid barrier of the one-launch Gram-Schmidt step: arrivals, generation
+  unsigned* bar = nullptr;    // [3] grid barrier of the one-launch Gram-Schmidt step: arrivals, generation, ran out
   int *err = nullptr, *err_dev = nullptr;  // mapped host word: a grid barrier ran out
+  unsigned spins = 0;         // bound of a barrier's wait
   int sms = 0, smem = 0;
 };
 
@@ -100,8 +101,10 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
   fv_system* sm = const_cast<fv_system*>(s);
   if (!sm->kry) sm->kry = new Krylov();
   KrylovT<T>& k = kt<T>(sm->kry);
+  k.spins = s->wait_limit;
   if (k.m >= m && k.n == s->n) return FV_OK;
   free_kt(k);
+  k.spins = s->wait_limit;
   if (sizeof(T) == 4) ++sm->kry->moves;
   k.m = m, k.n = s->n;
   const size_t n = (size_t)s->n;
@@ -111,7 +114,7 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
       cudaMalloc(&k.h, 3 * KMAX * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&k.ad, sizeof(ArnoldiDev)) != cudaSuccess || cudaMalloc(&k.ticket, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(k.ticket, 0, sizeof(unsigned)) != cudaSuccess ||
-      cudaMalloc(&k.bar, 2 * sizeof(unsigned)) != cudaSuccess || cudaMemset(k.bar, 0, 2 * sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&k.bar, 3 * sizeof(unsigned)) != cudaSuccess || cudaMemset(k.bar, 0, 3 * sizeof(unsigned)) != cudaSuccess ||
       cudaHostAlloc((void**)&k.err, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
       cudaHostGetDevicePointer((void**)&k.err_dev, k.err, 0) != cudaSuccess ||
       cudaMallocHost(&k.hhost, 3 * KMAX * sizeof(double)) != cudaSuccess) {
@@ -120,6 +123,33 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
   }
   *k.err = 0;
   return gs_limits<T>(k);
+}
+
+// After a synchronisation of st: whether a grid barrier of s's workspaces (either type) or of its coarse levels' ran out
+// since the last call.  The words are cleared and the barriers made usable again.
+static fv_status gs_failed(const fv_system* s, cudaStream_t st, bool* bad) {
+  auto check = [&](auto& k) -> fv_status {
+    if (!k.err || !*(volatile int*)k.err) return FV_OK;
+    *bad = true, *k.err = 0;
+    FV_CUDA(cudaMemsetAsync(k.bar, 0, 3 * sizeof(unsigned), st));
+    FV_CUDA(cudaStreamSynchronize(st));
+    return FV_OK;
+  };
+  fv_status rc;
+  for (; s; s = s->coarse)
+    if (s->kry && ((rc = check(s->kry->d)) || (rc = check(s->kry->f)))) return rc;
+  return FV_OK;
+}
+
+fv_status waits_failed(const fv_system* s, const char* where, cudaStream_t st) {
+  bool grid = false;
+  fv_status rc = gs_failed(s, st, &grid);
+  const bool sweep = sweep_failed(s);
+  if (rc) return rc;
+  if (grid || sweep)
+    return set_error(std::string(where) + (grid ? "a wait of the Gram-Schmidt steps ran out" : "a wait of the subdomain sweeps ran out")),
+           FV_ECUDA;
+  return FV_OK;
 }
 
 // ------------------------------------------------------------------ vector kernels
@@ -423,7 +453,6 @@ constexpr int GS_THREADS = 512;          // threads a block at most
 // converted to FP64 on the slow pipe (coarse level, 5 vectors: 24.6 us with 512 threads, see gs_step())
 __host__ __device__ constexpr int gs_threads(int nv, int es) { return es == 4 || nv > 16 ? GS_THREADS / 2 : GS_THREADS; }
 constexpr int GS_CHUNK = 8;              // values reduced together: [GS_CHUNK][GS_THREADS] doubles of shared memory
-constexpr unsigned GS_SPINS = 1u << 24;  // bound of a barrier's wait
 
 struct GsArgs {
   long long n, slice;   // elements; elements a block
@@ -437,16 +466,22 @@ struct GsArgs {
   ArnoldiDev* ad;       // device-driven solves
   unsigned* bar;
   int* err;
+  unsigned spins;
 };
 
-// all blocks (co-resident: cooperative launch) meet; bounded, a wait that runs out is reported through err
-__device__ __forceinline__ void grid_barrier(unsigned* bar, int* err) {
+// All blocks (co-resident: cooperative launch) meet.  The wait is bounded.  A block whose wait runs out goes on with
+// incomplete sums (every access stays in range), says so through err, and marks the barrier: later barriers, whose
+// count no longer fits, return at once, until the host has read err and reset the words (gs_failed).
+__device__ __forceinline__ void grid_barrier(unsigned* bar, int* err, unsigned spins) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned gen, cur;
+    unsigned gen, cur, lost;
     asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(gen) : "l"(bar + 1) : "memory");
+    asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(lost) : "l"(bar + 2) : "memory");
     __threadfence();
-    if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+    if (lost) {
+      *err = 1;
+    } else if (atomicAdd(bar, 1u) == gridDim.x - 1) {
       bar[0] = 0;
       __threadfence();
       atomicAdd(bar + 1, 1u);
@@ -454,8 +489,8 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, int* err) {
       unsigned t = 0;
       do {
         asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(bar + 1) : "memory");
-      } while (cur == gen && ++t < GS_SPINS);
-      if (cur == gen) *err = 1;
+      } while (cur == gen && ++t < spins);
+      if (cur == gen) *err = 1, atomicExch(bar + 2, 1u);
     }
     __threadfence();
   }
@@ -602,7 +637,7 @@ __global__ void __launch_bounds__(gs_threads(NV, sizeof(T)), 1) gs_kernel(GsArgs
     pass(std::true_type(), false, true);
     gs_reduce<NA, TH>(acc, NV, red, part);
     for (int q = 0; q < A.passes; ++q) {
-      grid_barrier(A.bar, A.err);
+      grid_barrier(A.bar, A.err, A.spins);
       gs_total<TH>(part, NV, tot);
       if (threadIdx.x < NV) {
         hs[threadIdx.x] = (T)tot[threadIdx.x];
@@ -620,7 +655,7 @@ __global__ void __launch_bounds__(gs_threads(NV, sizeof(T)), 1) gs_kernel(GsArgs
     pass(std::true_type(), false, false);
     gs_reduce<NA, TH>(acc, 1, red, part);
   }
-  grid_barrier(A.bar, A.err);
+  grid_barrier(A.bar, A.err, A.spins);
   gs_total<TH>(part, 1, tot);
   // one thread takes the square root and the reciprocal: on the FP64 pipe (16 cycles a warp instruction) every
   // warp doing so cost more than a pass over the basis
@@ -821,7 +856,7 @@ static fv_status gs_step(const KrylovT<T>& k, int nv, long long n, const T* w, T
     a.keep = nv > 0 && n % Vec16<T>::L == 0 && smem + keep <= (size_t)k.smem;
     if (a.keep) smem += keep;
     a.n = n, a.passes = nv > 0 ? passes : 0, a.start = nv == 0, a.last = last, a.gj = nv - 1;
-    a.part = k.part, a.h = k.h, a.ad = ad, a.bar = k.bar, a.err = k.err_dev;
+    a.part = k.part, a.h = k.h, a.ad = ad, a.bar = k.bar, a.err = k.err_dev, a.spins = k.spins;
     const T* V = nv > 0 ? k.V : w;
     void* args[] = {&a, &V, &w, &vout};
     FV_CUDA(cudaLaunchCooperativeKernel(gs_kernel_of<T>(nv, std::make_integer_sequence<int, KMAX>{}), dim3(blocks),
@@ -1152,8 +1187,7 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
     if (!std::isfinite(beta)) nan = true;
     if (breakdown) break;
   }
-  if (*(volatile int*)k.err) return *k.err = 0, set_error("fv_gmres_solve: a grid barrier ran out"), FV_ECUDA;
-  if (sweep_failed(s)) return set_error("fv_gmres_solve: a wait of the subdomain sweeps ran out"), FV_ECUDA;
+  if ((rc = waits_failed(s, "fv_gmres_solve: ", st))) return rc;
   const bool conv = !nan && beta <= target;
   if (stats) {
     stats->iters = its;
