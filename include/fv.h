@@ -39,7 +39,7 @@ typedef int fv_status;
 #define FV_OK 0
 #define FV_EINVAL (-1)      /* bad argument (null handle, bad size, odd grid for two levels) */
 #define FV_ENOMEM (-2)      /* device allocation failed */
-#define FV_ECUDA (-3)       /* a CUDA call failed; the message names it */
+#define FV_ECUDA (-3)       /* a CUDA call failed, or a bounded wait in a kernel ran out; the message names it */
 #define FV_ENOCONV (-4)     /* GMRES hit max_it before the tolerance; x holds the last iterate */
 #define FV_EBREAKDOWN (-5)  /* zero pivot in ILU(0) */
 #define FV_ENAN (-6)        /* NaN/Inf residual; x holds the last finite iterate */
@@ -173,7 +173,11 @@ fv_status fv_apply_op_fp32(const fv_system* s, const float* x, float* y, void* s
 fv_status fv_apply_op_noalloc(const fv_system* s, const double* x, double* y, void* stream);
 
 /* z = M^{-1} r (eqn:onelevel or eqn:twolevel per the system's pc).
- * r, z: device FP64, n values each, must not overlap. */
+ * r, z: device FP64, n values each, must not overlap.  The call returns
+ * before its kernels have finished where no coarse FP64 solve is part of it: a
+ * bounded wait that runs out in them is reported by the next application or
+ * solve on the system, which then returns FV_ECUDA without having begun (x and
+ * z as they were). */
 fv_status fv_precond_apply(const fv_system* s, const double* r, double* z, void* stream);
 
 /* Restarted right-preconditioned flexible GMRES(restart) (paper Sec. 3.3):

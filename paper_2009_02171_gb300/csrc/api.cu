@@ -179,6 +179,7 @@ fv_status fv_apply_op_noalloc(const fv_system* s, const double* x, double* y, vo
 
 fv_status fv_precond_apply(const fv_system* s, const double* r, double* z, void* stream) {
   if (!s || !r || !z || r == z) return set_error("fv_precond_apply: bad argument"), FV_EINVAL;
+  if (fv_status rc = waits_failed(s, "fv_precond_apply: not begun, in an earlier call ", (cudaStream_t)stream)) return rc;
   s->last_inner = 0;
   return precond_apply(s, r, z, (cudaStream_t)stream);
 }

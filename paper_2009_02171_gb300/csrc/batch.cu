@@ -648,6 +648,7 @@ fv_status gmres_batch(const fv_system* s, int nrhs, const double* B, double* X, 
     return FV_OK;
   };
   if ((rc = fetch_state())) return rc;
+  if ((rc = waits_failed(s, "fv_gmres_solve_batch: not begun, in an earlier call ", st))) return rc;
   auto any_active = [&]() {
     for (int t = 0; t < nrhs; ++t)
       if (!bw->arn_host[t].done) return true;

@@ -272,7 +272,7 @@ fv_status gmres(const fv_system* s, const double* b, double* x, const fv_gmres_o
                 cudaStream_t st, bool inner);
 void free_krylov(Krylov* k);
 unsigned long long inner_buffers(const fv_system* s);
-// after a synchronisation: FV_ECUDA if a bounded wait of s or of its coarse levels ran out since the last call
+// FV_ECUDA if a bounded wait of s or of its coarse levels ran out in work that has finished, since the last call
 fv_status waits_failed(const fv_system* s, const char* where, cudaStream_t st);
 void free_batch(BatchWork* b);
 fv_status axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st);

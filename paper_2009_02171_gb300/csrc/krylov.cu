@@ -125,8 +125,8 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
   return gs_limits<T>(k);
 }
 
-// After a synchronisation of st: whether a grid barrier of s's workspaces (either type) or of its coarse levels' ran out
-// since the last call.  The words are cleared and the barriers made usable again.
+// Whether a grid barrier of s's workspaces (either type) or of its coarse levels' ran out, in work on st, since the last
+// call.  The words are cleared and the barriers made usable again.
 static fv_status gs_failed(const fv_system* s, cudaStream_t st, bool* bad) {
   auto check = [&](auto& k) -> fv_status {
     if (!k.err || !*(volatile int*)k.err) return FV_OK;
@@ -1119,6 +1119,8 @@ static fv_status gmres_t(const fv_system* s, const T* b, T* x, const fv_gmres_op
   if ((rc = apply_t<T>(s, x, k.r, st, b))) return rc;
   double beta;
   if ((rc = norm2<T>(k, n, k.r, k.V, st, &beta))) return rc;
+  // the stream has been waited for and x is as it was: what fv_precond_apply calls before this one left
+  if (!inner && (rc = waits_failed(s, "fv_gmres_solve: not begun, in an earlier call ", st))) return rc;
   const double r0 = beta, target = std::max(o->atol, o->rtol * r0);
   int its = 0;
   bool nan = !std::isfinite(beta);

@@ -49,3 +49,30 @@ def test_a_barrier_that_runs_out_fails_the_solve_and_no_later_one(prec, levels, 
     for q in (s, fresh):
         fv.fv_free_system(q)
     fv.fv_free_grid(g)
+
+
+@pytest.mark.parametrize('batch', [False, True])
+def test_an_application_that_failed_is_reported_before_the_next_call_begins(batch):
+    from paper_2009_02171_gb300 import fv
+    g = fv.fv_build_grid(16, 12)
+    s, b = _system(fv, g, 1, 1)
+    _limit(fv, s, 1)
+    z = fv.fv_precond_apply(s, b, torch.empty_like(b))  # returns before its kernels have finished
+    torch.cuda.synchronize()
+    _limit(fv, s, DEFAULT)
+    x = torch.full_like(b, 0.5)
+    solve = ((lambda: fv.fv_gmres_solve_batch(s, b[None], x[None], rtol=1e-8)[0]) if batch else
+             (lambda: fv.fv_gmres_solve(s, b, x, rtol=1e-8)))
+    with pytest.raises(fv.FvError, match='not begun, in an earlier call'):
+        solve()
+    assert (x == 0.5).all()
+    assert solve().converged
+    _limit(fv, s, 1)
+    fv.fv_precond_apply(s, b, z)
+    torch.cuda.synchronize()
+    z.fill_(0.5)
+    with pytest.raises(fv.FvError, match='not begun, in an earlier call'):
+        fv.fv_precond_apply(s, b, z)
+    assert (z == 0.5).all()
+    fv.fv_free_system(s)
+    fv.fv_free_grid(g)
