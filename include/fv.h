@@ -208,7 +208,7 @@ fv_status fv_gmres_solve(const fv_system* s, const double* b, double* x, const f
  * The preconditioner is the system's one-level RAS (levels = 1 only), with
  * FP32 subdomain solves when the system was assembled with FV_PREC_FP32,
  * one launch over all (subdomain, right-hand side) pairs.  Subdomains too wide
- * for that (above 384 rows in a wavefront's window): every factor loaded is
+ * for that (above 384 cells in a wavefront): every factor loaded is
  * applied to a group of right-hand sides (the group size is tuned by timing
  * on the first call for a given nrhs), in one persistent launch a direction
  * that takes subdomains largest first.

@@ -10,7 +10,8 @@
 // chain short and everything else off it:
 //  * A thread owns rows of cells along i.  Rows (j, k) are ranked by s = 2 j + k, so the rows active in a step
 //    (0 <= L - s < nx) are consecutive ranks: warps are full or idle, and the operands of a step, packed in rank
-//    order, sit at rank + offset(L).  Thread t runs the ranks t, t + T, t + 2 T, ..., T the widest window.
+//    order, sit at rank + offset(L).  Thread t runs the ranks t, t + T, t + 2 T, ..., T at least the widest step: a
+//    thread has finished its row before its next one begins.
 //  * Of a cell's five neighbours, (i -+ 1, j, k) is the thread's own last value and the three in row (j -+ 1, k)
 //    are that row's last three values, of which two are already in registers: a step reads two values from a
 //    two-deep ring in shared memory, does two dependent multiply-adds a component, stores one and meets a barrier.
@@ -35,7 +36,8 @@ namespace fv {
 namespace {
 
 constexpr int SLOTS = 8;             // chunks of the operand ring
-constexpr int MAX_ROWS = 384;        // widest window of rows a CTA takes (threads of the solve)
+constexpr int MAX_ROWS = 384;        // cells of the widest step a CTA takes (threads of the solve)
+constexpr int NEAR_TABLE = 48 << 10; // largest step and row tables kept in shared memory (WIDE: the steps alone)
 constexpr int PRODUCERS = 64;        // one warp for the operands, one for the right-hand side
 constexpr unsigned WAIT_TRIES = 1u << 22;
 
@@ -199,8 +201,10 @@ struct Cell {
 // cells a chunk: the ring holds SLOTS of them
 __host__ __device__ constexpr int chunk_log(int kind) { return kind == FV_VTBE ? 6 : 7; }
 
-// LOCS: the forward result of the box stays in shared memory
-template <int DG, int LG, bool LOCS, class T, class V, class FT>
+// LOCS: the forward result of the box stays in shared memory.  WIDE: the row table is read from global memory, a row
+// ahead, and a row may begin the step after its thread's last one ended (as a test in the common variant that cost 1 to
+// 5 % of a step: registers)
+template <int DG, int LG, bool LOCS, bool WIDE, class T, class V, class FT>
 __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, int c0, T* loc, const V* __restrict__ r,
                                            V* __restrict__ z, unsigned char* smem) {
   using LF = Lay<DG, FT, true>;
@@ -245,7 +249,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
   }
   for (int e = tid; e < 2 * NC * RV; e += blockDim.x) ring[e] = T(0);
   for (int e = tid; e <= levels; e += blockDim.x) steps[e] = A.steps[sh.steps + e];
-  for (int e = tid; e < rows; e += blockDim.x) row[e] = A.rows[sh.table + e];
+  if constexpr (!WIDE)
+    for (int e = tid; e < rows; e += blockDim.x) row[e] = A.rows[sh.table + e];
   __syncthreads();
 
   if (tid >= NC + 32) {  // ------------------------------------------------ right-hand side warp
@@ -330,11 +335,17 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
   const T *jrow, *krow;  // the neighbour rows' places in the ring
   T own[DG], h1[DG], h2[DG];
   constexpr int OFF = -0x10000000;  // i of a thread without a row
-  // row `rk` from step L on (sh0: bit position of the direction's pair of neighbours)
-  auto take_row = [&](int rk, int L, int sh0) {
+  unsigned long long ahead = 0;  // WIDE: the table's entry of the thread's next row
+  auto look_ahead = [&](int rk) {
+    if constexpr (WIDE) ahead = rk >= 0 && rk < rows ? __ldg(A.rows + sh.table + rk) : 0;
+  };
+  // row `rk` from step L on (sh0: bit position of the direction's pair of neighbours), the thread's next one after
+  // `by` ranks
+  auto take_row = [&](int rk, int L, int sh0, int by) {
     rank = rk;
     const bool on = rk >= 0 && rk < rows && !dead;
-    const unsigned long long w = on ? row[rk] : 0;
+    const unsigned long long w = WIDE ? ahead : on ? row[rk] : 0;
+    look_ahead(rk + by);
     i = on ? L - (int)(w & 0xffff) : OFF;
     jrow = ring + ((int)(w >> sh0) & 0xfff) * RV, krow = ring + ((int)(w >> (sh0 + 12)) & 0xfff) * RV;
 #pragma unroll
@@ -358,7 +369,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
         for (int a = 0; a < DG; ++a) q.y[a] = (T) reinterpret_cast<const V*>(ybuf)[a * CAP + idx];
       }
     };
-    take_row(tid, 0, 16);
+    look_ahead(tid);
+    take_row(tid, 0, 16, NC);
     int2 cur = steps[0], nxt = steps[1];
     fetch(cur);
     int free_at = min(CH, nc);
@@ -399,7 +411,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
         free_at = min((freed + 1) << LG, nc);
       }
       cur = nxt;
-      if (++i == nx) take_row(rank + NC, L + 1, 16);
+      if (++i == nx) {
+        take_row(rank + NC, L + 1, 16, NC);
+        // a row that begins with the next step (a window wider than T) reads (0, j - 1, k) of step L - 1 here; others
+        // wait a step at i = -1, which reads it
+        if (WIDE && i == 0) R::load(jrow + last, h1);
+      }
       nxt = steps[min(L + 2, levels)];
       if (L + 1 < levels) fetch(cur);
       step_barrier(NC);
@@ -429,7 +446,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
       }
     };
     // the last rank of this thread
-    take_row(tid < rows ? tid + (rows - 1 - tid) / NC * NC : -1, levels - 1, 40);
+    const int top = tid < rows ? tid + (rows - 1 - tid) / NC * NC : -1;
+    look_ahead(top);
+    take_row(top, levels - 1, 40, -NC);
     int2 cur = steps[levels - 1], nxt = steps[max(levels - 2, 0)];
     int begin = levels > 1 ? nxt.y : 0;  // first cell of the step whose operands are held
     fetch(cur, begin);
@@ -472,7 +491,10 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
         free_at = (2 * nch - 1 - freed) << LG;
       }
       cur = nxt;
-      if (--i == -1) take_row(rank - NC, L - 1, 40);
+      if (--i == -1) {
+        take_row(rank - NC, L - 1, 40, -NC);
+        if (WIDE && i == nx - 1) R::load(jrow + last, h1);  // (nx - 1, j + 1, k) of step L + 1
+      }
       nxt = steps[max(L - 2, 0)];
       begin = L > 1 ? nxt.y : 0;
       if (L > 0) fetch(cur, begin);
@@ -485,7 +507,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
 }
 
 // grid: x = component group * boxes + box in decreasing size (the heavier group first), y = right-hand side
-template <class T, class V, class FT, int KIND, bool LOCS>
+template <class T, class V, class FT, int KIND, bool LOCS, bool WIDE>
 __global__ void __launch_bounds__(MAX_ROWS + PRODUCERS, sizeof(T) == 8 && KIND == FV_VTBE ? 1 : 2)
     ras_stream_kernel(const __grid_constant__ SweepArgs A, const V* __restrict__ r, V* __restrict__ z) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -495,12 +517,12 @@ __global__ void __launch_bounds__(MAX_ROWS + PRODUCERS, sizeof(T) == 8 && KIND =
   r += rhs * A.rs, z += rhs * A.zs;
   const int g = (int)blockIdx.x >= A.count, sd = A.lpt[blockIdx.x - g * A.count];
   if constexpr (KIND == FV_VTBE) {
-    if (g == 0) sweep_body<4, LG, LOCS, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
-    else sweep_body<3, LG, LOCS, T, V, FT>(A, sd, 1, 4, loc, r, z, smem);
+    if (g == 0) sweep_body<4, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
+    else sweep_body<3, LG, LOCS, WIDE, T, V, FT>(A, sd, 1, 4, loc, r, z, smem);
   } else if constexpr (sizeof(T) == 8) {
-    sweep_body<1, LG, LOCS, T, V, FT>(A, sd, g, g, loc, r, z, smem);
+    sweep_body<1, LG, LOCS, WIDE, T, V, FT>(A, sd, g, g, loc, r, z, smem);
   } else {
-    sweep_body<2, LG, LOCS, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
+    sweep_body<2, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
   }
 }
 
@@ -593,16 +615,19 @@ fv_status launch(const fv_system* s, int nrhs, const V* r, long long rs, V* z, l
   SweepArgs a{(const Shape*)q.shapes, q.shape_of, (const int2*)q.steps, q.rows, S.lpt, q.soff, {q.fw[0], q.fw[1]},
               {q.bw[0], q.bw[1]}, q.gather, loc, q.err_dev, q.sT, s->grid->h.N, rs, zs, S.count, q.T, q.table_bytes};
   const dim3 grid(q.groups * S.count, nrhs);
-  if (q.loc_smem) ras_stream_kernel<T, V, FT, KIND, true><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
-  else ras_stream_kernel<T, V, FT, KIND, false><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
+  if (q.wide) ras_stream_kernel<T, V, FT, KIND, false, true><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
+  else if (q.loc_smem) ras_stream_kernel<T, V, FT, KIND, true, false><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
+  else ras_stream_kernel<T, V, FT, KIND, false, false><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
   FV_CUDA(cudaGetLastError());
   return FV_OK;
 }
 
 template <class T, class V, class FT, int KIND>
 fv_status allow_smem_k(int limit) {
-  FV_CUDA(cudaFuncSetAttribute(ras_stream_kernel<T, V, FT, KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  FV_CUDA(cudaFuncSetAttribute(ras_stream_kernel<T, V, FT, KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  for (const void* f : {(const void*)ras_stream_kernel<T, V, FT, KIND, true, false>,
+                        (const void*)ras_stream_kernel<T, V, FT, KIND, false, false>,
+                        (const void*)ras_stream_kernel<T, V, FT, KIND, false, true>})
+    FV_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   return FV_OK;
 }
 template <class T, class V, class FT>
@@ -612,9 +637,12 @@ fv_status allow_smem(int d, int limit) {
 
 }  // namespace
 
-// Builds the streams of s when every box fits the scheme: its widest window of rows has a thread for every row
-// (MAX_ROWS), and a ring of SLOTS chunks that holds a whole step fits in shared memory.  *used = 0: the caller
-// keeps the general sweeps.
+// Builds the streams of s when every box fits the scheme: its widest step has a thread for every cell (MAX_ROWS), and
+// a ring of SLOTS chunks that holds a whole step fits in shared memory.  *used = 0: the caller keeps the general sweeps,
+// 1.2 to 5 times slower where both can run (us, general against these: PPBE FP32 boxes of 36x36x21 cells 357, 156,
+// 48x48x16 516, 205, 4x96x96 1689, 423; VTBE FP32 24x24x32 1067, 322; VTBE FP64 24x24x32 1736, 596).  Rows are held one
+// step before they begin where MAX_ROWS threads cover such a window (to 36x36x20 cells: a window of 384); the boxes above
+// have steps of 376 to 384 cells and windows to 396, or more rows than shared memory holds a table of, and run WIDE.
 fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::vector<long long>& cell_off, int* used) {
   *used = 0;
   Subdomains& S = s->subs;
@@ -629,7 +657,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   std::vector<int2> steps;
   std::vector<unsigned long long> rows;
   std::vector<std::array<int, 3>> boxes;
-  int window = 1, widest = 1, max_table = 0;
+  int window = 1, widest = 1, max_table = 0, max_steps = 0;
   long long max_nc = 0;
   for (int b = 0; b < S.count; ++b) {
     const std::array<int, 3> box{dims[3 * b], dims[3 * b + 1], dims[3 * b + 2]};
@@ -652,7 +680,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
         steps.push_back(make_int2(cells - from, cells + n));
         cells += n;
         widest = std::max(widest, n);
-        // a row is held one step longer than it is active (forward: before, backward: after)
+        // a row held one step longer than it is active (forward: before, backward: after)
         window = std::max(window, std::max(upto(L + 1) - upto(L - nx), upto(L) - upto(L - nx - 1)));
       }
       steps.push_back(make_int2(0, cells));
@@ -660,11 +688,13 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
       shapes.push_back(sh), boxes.push_back(box);
       max_nc = std::max<long long>(max_nc, sh.nc);
       max_table = std::max(max_table, (sh.levels + 1 + sh.rows) * 8);
+      max_steps = std::max(max_steps, (sh.levels + 1) * 8);
     }
     shape_of[b] = it->second;
   }
-  if (window > MAX_ROWS || max_table > 48 * 1024) return FV_OK;
-  q.T = (window + 31) / 32 * 32;
+  if (widest > MAX_ROWS) return FV_OK;
+  q.T = (std::min(window, MAX_ROWS) + 31) / 32 * 32;
+  q.wide = window > MAX_ROWS || max_table > NEAR_TABLE;
   for (size_t m = 0; m < shapes.size(); ++m) {
     const Shape& sh = shapes[m];
     const int ny = boxes[m][1], nz = boxes[m][2];
@@ -685,7 +715,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   FV_CUDA(cudaGetDevice(&dev));
   FV_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  q.table_bytes = (max_table + 127) / 128 * 128;
+  q.table_bytes = ((q.wide ? max_steps : max_table) + 127) / 128 * 128;
   const int dg = d == 7 ? 4 : S.fp32 ? 2 : 1;  // the wider group
   // right-hand sides are staged in the vectors' type; a batch on FP32 factors stages FP64 (one level only)
   const size_t per_cell = std::max(fw[0], bw[0]) + (size_t)dg * (s->pc.levels == 1 && !S.bf16 ? 8 : es);
@@ -696,7 +726,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   // the forward result stays in shared memory where that costs no CTA an SM would otherwise hold
   const int tasks = (q.groups * S.count + sms - 1) / sms, sm_bytes = limit + 1024;
   const int fit = std::min(sm_bytes / (int)(q.smem + 1024), d == 7 && !S.fp32 ? 1 : std::max(2, 1024 / (q.T + PRODUCERS)));
-  q.loc_smem = q.smem + loc <= (size_t)limit && sm_bytes / (int)(q.smem + loc + 1024) >= std::min(tasks, fit);
+  q.loc_smem = !q.wide && q.smem + loc <= (size_t)limit && sm_bytes / (int)(q.smem + loc + 1024) >= std::min(tasks, fit);
   if (q.loc_smem) q.smem += loc;
   const long long CH = 1LL << q.ch_log;
   std::vector<long long> so(S.count + 1, 0);
