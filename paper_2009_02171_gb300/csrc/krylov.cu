@@ -479,9 +479,10 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, int* err, unsigned s
     asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(gen) : "l"(bar + 1) : "memory");
     asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(lost) : "l"(bar + 2) : "memory");
     __threadfence();
+    const unsigned before = atomicAdd(bar, 1u);  // the marks are read beside it, not before it
     if (lost) {
       *err = 1;
-    } else if (atomicAdd(bar, 1u) == gridDim.x - 1) {
+    } else if (before == gridDim.x - 1) {
       bar[0] = 0;
       __threadfence();
       atomicAdd(bar + 1, 1u);
