@@ -103,8 +103,7 @@ struct SweepStream {
   void *shapes = nullptr, *steps = nullptr;  // tables of the distinct box shapes
   int* shape_of = nullptr;
   unsigned long long* rows = nullptr;
-  int groups = 0, T = 0, ch_log = 0, loc_smem = 0, table_bytes = 0;  // T: threads of the solve; cells a chunk (log2)
-  int wide = 0;                      // 1: a window of rows wider than T, or a row table too large for shared memory
+  int groups = 0, T = 0, ch_log = 0, variant = 0, table_bytes = 0;  // T: threads of the solve; cells a chunk (log2)
   size_t smem = 0;
   int *err = nullptr, *err_dev = nullptr;  // mapped host word: a wait of the sweep ran out
 };

@@ -16,7 +16,7 @@
 //    are that row's last three values, of which two are already in registers: a step reads two values from a
 //    two-deep ring in shared memory, does two dependent multiply-adds a component, stores one and meets a barrier.
 //  * Operands are streamed.  A cell's factors and its grid cell are packed into 16-byte words, chunk by chunk; one
-//    thread keeps a ring of SLOTS chunks filled with cp.async.bulk, ahead of the steps by as much as the ring
+//    thread keeps a ring of eight (small: four) chunks filled with cp.async.bulk, ahead of the steps by as much as the ring
 //    holds, and a second warp gathers the right-hand side through the cell map (forward) or reads the forward
 //    result back (backward) with cp.async, completion counted by mbarriers.
 // Positions outside the box have exactly zero factors (assembly writes zero there and the factorization never
@@ -35,7 +35,6 @@ namespace fv {
 
 namespace {
 
-constexpr int SLOTS = 8;             // chunks of the operand ring
 constexpr int MAX_ROWS = 384;        // cells of the widest step a CTA takes (threads of the solve)
 constexpr int NEAR_TABLE = 48 << 10; // largest step and row tables kept in shared memory (WIDE: the steps alone)
 constexpr int PRODUCERS = 64;        // one warp for the operands, one for the right-hand side
@@ -198,20 +197,26 @@ struct Cell {
   __device__ __forceinline__ int cell() const { return (int)w[L::NFW]; }
 };
 
-// cells a chunk: the ring holds SLOTS of them
-__host__ __device__ constexpr int chunk_log(int kind) { return kind == FV_VTBE ? 6 : 7; }
+// How a system's sweeps run: ring and row table as below, forward results in global memory or (LOCS) shared memory
+enum Variant { GLOBAL_LOC, SHARED_LOC, WIDE_ROWS, SMALL_GLOBAL_LOC, SMALL_SHARED_LOC, VARIANTS };
+// chunks of the operand ring (log2), cells a chunk (log2)
+__host__ __device__ constexpr int slots_log(int kind, bool small) { return small && kind == FV_VTBE ? 2 : 3; }
+__host__ __device__ constexpr int chunk_log(int kind, bool small) { return small ? 5 : kind == FV_VTBE ? 6 : 7; }
+constexpr int SMALL_STEP = 64;  // widest step of the small ring: it holds three and more steps ahead of the solve
+constexpr int max_threads(int var) { return (var >= SMALL_GLOBAL_LOC ? 2 * SMALL_STEP : MAX_ROWS) + PRODUCERS; }
+constexpr int min_ctas(int var, bool heavy) { return var >= SMALL_GLOBAL_LOC ? (heavy ? 2 : 4) : heavy ? 1 : 2; }
 
 // LOCS: the forward result of the box stays in shared memory.  WIDE: the row table is read from global memory, a row
 // ahead, and a row may begin the step after its thread's last one ended (as a test in the common variant that cost 1 to
 // 5 % of a step: registers)
-template <int DG, int LG, bool LOCS, bool WIDE, class T, class V, class FT>
+template <int DG, int SL, int LG, bool LOCS, bool WIDE, class T, class V, class FT>
 __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, int c0, T* loc, const V* __restrict__ r,
                                            V* __restrict__ z, unsigned char* smem) {
   using LF = Lay<DG, FT, true>;
   using LB = Lay<DG, FT, false>;
   constexpr int RV = DG == 3 ? 4 : DG;  // values a cell holds in the step ring
   using R = RingVec<DG, T>;
-  constexpr int CH = 1 << LG, CAP = SLOTS << LG;
+  constexpr int SLOTS = 1 << SL, CH = 1 << LG, CAP = SLOTS << LG;
   const int NC = A.T, tid = threadIdx.x;
   const Shape sh = A.shapes[A.shape_of[sd]];
   const int nx = sh.nx, nc = sh.nc, levels = sh.levels, rows = sh.rows;
@@ -272,7 +277,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
         const int n = n0 + u;
         if (n >= nch || dead) break;
         const int slot = n & (SLOTS - 1), b = (slot << LG) + lane;
-        if (n >= SLOTS) bar_wait(empty + 8 * slot, ((n >> 3) - 1) & 1, dead, A.err);
+        if (n >= SLOTS) bar_wait(empty + 8 * slot, ((n >> SL) - 1) & 1, dead, A.err);
         if (dead) break;
 #pragma unroll
         for (int e = 0; e < PL; ++e) {
@@ -289,7 +294,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
       bar_wait(fdone, 0, dead, A.err);
       for (int n = nch; n < 2 * nch && !dead; ++n) {
         const int slot = n & (SLOTS - 1), b = slot << LG;
-        if (n >= SLOTS) bar_wait(empty + 8 * slot, ((n >> 3) - 1) & 1, dead, A.err);
+        if (n >= SLOTS) bar_wait(empty + 8 * slot, ((n >> SL) - 1) & 1, dead, A.err);
         if (dead) break;
         constexpr int PER = 16 / sizeof(T);
         const T* src = loc + ((2 * nch - 1 - n) << LG);
@@ -307,12 +312,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
     if (tid > NC) return;
     int n = first;
     for (; n < 2 * nch; ++n) {
-      bar_wait(empty + 8 * (n & (SLOTS - 1)), ((n >> 3) - 1) & 1, dead, A.err);
+      bar_wait(empty + 8 * (n & (SLOTS - 1)), ((n >> SL) - 1) & 1, dead, A.err);
       if (dead) break;
       load_chunk(n);
     }
     bool late = false;
-    for (int q = max(0, n - SLOTS); q < n; ++q) bar_wait(full + 8 * (q & (SLOTS - 1)), (q >> 3) & 1, late, A.err);
+    for (int q = max(0, n - SLOTS); q < n; ++q) bar_wait(full + 8 * (q & (SLOTS - 1)), (q >> SL) & 1, late, A.err);
     return;
   }
 
@@ -320,7 +325,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
   int waited = 0;  // chunks that have been waited for
   auto await = [&](int upto, bool y) {
     while (waited < upto) {
-      const int slot = waited & (SLOTS - 1), par = (waited >> 3) & 1;
+      const int slot = waited & (SLOTS - 1), par = (waited >> SL) & 1;
       bar_wait(full + 8 * slot, par, dead, A.err);
       if (y) bar_wait(yfull + 8 * slot, par, dead, A.err);
       ++waited;
@@ -507,22 +512,23 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& A, int sd, int g, in
 }
 
 // grid: x = component group * boxes + box in decreasing size (the heavier group first), y = right-hand side
-template <class T, class V, class FT, int KIND, bool LOCS, bool WIDE>
-__global__ void __launch_bounds__(MAX_ROWS + PRODUCERS, sizeof(T) == 8 && KIND == FV_VTBE ? 1 : 2)
+template <class T, class V, class FT, int KIND, int VAR>
+__global__ void __launch_bounds__(max_threads(VAR), min_ctas(VAR, sizeof(T) == 8 && KIND == FV_VTBE))
     ras_stream_kernel(const __grid_constant__ SweepArgs A, const V* __restrict__ r, V* __restrict__ z) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int rhs = blockIdx.y;
-  constexpr int D = KIND == FV_VTBE ? 7 : 2, LG = chunk_log(KIND);
+  constexpr int D = KIND == FV_VTBE ? 7 : 2, SL = slots_log(KIND, VAR >= SMALL_GLOBAL_LOC), LG = chunk_log(KIND, VAR >= SMALL_GLOBAL_LOC);
+  constexpr bool LOCS = VAR == SHARED_LOC || VAR == SMALL_SHARED_LOC, WIDE = VAR == WIDE_ROWS;
   T* const loc = (T*)A.loc + (size_t)rhs * D * A.sT;
   r += rhs * A.rs, z += rhs * A.zs;
   const int g = (int)blockIdx.x >= A.count, sd = A.lpt[blockIdx.x - g * A.count];
   if constexpr (KIND == FV_VTBE) {
-    if (g == 0) sweep_body<4, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
-    else sweep_body<3, LG, LOCS, WIDE, T, V, FT>(A, sd, 1, 4, loc, r, z, smem);
+    if (g == 0) sweep_body<4, SL, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
+    else sweep_body<3, SL, LG, LOCS, WIDE, T, V, FT>(A, sd, 1, 4, loc, r, z, smem);
   } else if constexpr (sizeof(T) == 8) {
-    sweep_body<1, LG, LOCS, WIDE, T, V, FT>(A, sd, g, g, loc, r, z, smem);
+    sweep_body<1, SL, LG, LOCS, WIDE, T, V, FT>(A, sd, g, g, loc, r, z, smem);
   } else {
-    sweep_body<2, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
+    sweep_body<2, SL, LG, LOCS, WIDE, T, V, FT>(A, sd, 0, 0, loc, r, z, smem);
   }
 }
 
@@ -609,36 +615,42 @@ int group_bytes(int d, size_t (&fw)[2], size_t (&bw)[2]) {  // the number of gro
 }
 
 template <class T, class V, class FT, int KIND>
+const void* stream_kernel(int var) {
+  static const void* const table[VARIANTS] = {
+      (const void*)ras_stream_kernel<T, V, FT, KIND, GLOBAL_LOC>, (const void*)ras_stream_kernel<T, V, FT, KIND, SHARED_LOC>,
+      (const void*)ras_stream_kernel<T, V, FT, KIND, WIDE_ROWS>, (const void*)ras_stream_kernel<T, V, FT, KIND, SMALL_GLOBAL_LOC>,
+      (const void*)ras_stream_kernel<T, V, FT, KIND, SMALL_SHARED_LOC>};
+  return table[var];
+}
+
+template <class T, class V, class FT>
+const void* kernel_of(int d, int var) {
+  return d == 7 ? stream_kernel<T, V, FT, FV_VTBE>(var) : stream_kernel<T, V, FT, FV_PPBE>(var);
+}
+
+template <class T, class V, class FT, int KIND>
 fv_status launch(const fv_system* s, int nrhs, const V* r, long long rs, V* z, long long zs, void* loc, cudaStream_t st) {
   const Subdomains& S = s->subs;
   const SweepStream& q = S.st;
   SweepArgs a{(const Shape*)q.shapes, q.shape_of, (const int2*)q.steps, q.rows, S.lpt, q.soff, {q.fw[0], q.fw[1]},
               {q.bw[0], q.bw[1]}, q.gather, loc, q.err_dev, q.sT, s->grid->h.N, rs, zs, S.count, q.T, q.table_bytes};
-  const dim3 grid(q.groups * S.count, nrhs);
-  if (q.wide) ras_stream_kernel<T, V, FT, KIND, false, true><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
-  else if (q.loc_smem) ras_stream_kernel<T, V, FT, KIND, true, false><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
-  else ras_stream_kernel<T, V, FT, KIND, false, false><<<grid, q.T + PRODUCERS, q.smem, st>>>(a, r, z);
-  FV_CUDA(cudaGetLastError());
+  void* args[] = {&a, &r, &z};
+  FV_CUDA(cudaLaunchKernel(stream_kernel<T, V, FT, KIND>(q.variant), dim3(q.groups * S.count, nrhs), dim3(q.T + PRODUCERS), args,
+                           q.smem, st));
   return FV_OK;
 }
 
-template <class T, class V, class FT, int KIND>
-fv_status allow_smem_k(int limit) {
-  for (const void* f : {(const void*)ras_stream_kernel<T, V, FT, KIND, true, false>,
-                        (const void*)ras_stream_kernel<T, V, FT, KIND, false, false>,
-                        (const void*)ras_stream_kernel<T, V, FT, KIND, false, true>})
-    FV_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
-  return FV_OK;
-}
 template <class T, class V, class FT>
 fv_status allow_smem(int d, int limit) {
-  return d == 7 ? allow_smem_k<T, V, FT, FV_VTBE>(limit) : allow_smem_k<T, V, FT, FV_PPBE>(limit);
+  for (int var = 0; var < VARIANTS; ++var)
+    FV_CUDA(cudaFuncSetAttribute(kernel_of<T, V, FT>(d, var), cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+  return FV_OK;
 }
 
 }  // namespace
 
 // Builds the streams of s when every box fits the scheme: its widest step has a thread for every cell (MAX_ROWS), and
-// a ring of SLOTS chunks that holds a whole step fits in shared memory.  *used = 0: the caller keeps the general sweeps,
+// an operand ring that holds a whole step fits in shared memory.  *used = 0: the caller keeps the general sweeps,
 // 1.2 to 5 times slower where both can run (us, general against these: PPBE FP32 boxes of 36x36x21 cells 357, 156,
 // 48x48x16 516, 205, 4x96x96 1689, 423; VTBE FP32 24x24x32 1067, 322; VTBE FP64 24x24x32 1736, 596).  Rows are held one
 // step before they begin where MAX_ROWS threads cover such a window (to 36x36x20 cells: a window of 384); the boxes above
@@ -694,7 +706,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   }
   if (widest > MAX_ROWS) return FV_OK;
   q.T = (std::min(window, MAX_ROWS) + 31) / 32 * 32;
-  q.wide = window > MAX_ROWS || max_table > NEAR_TABLE;
+  const bool wide = window > MAX_ROWS || max_table > NEAR_TABLE;
   for (size_t m = 0; m < shapes.size(); ++m) {
     const Shape& sh = shapes[m];
     const int ny = boxes[m][1], nz = boxes[m][2];
@@ -715,23 +727,48 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   FV_CUDA(cudaGetDevice(&dev));
   FV_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  q.table_bytes = ((q.wide ? max_steps : max_table) + 127) / 128 * 128;
+  fv_status rc;
+  if (S.bf16) rc = allow_smem<float, float, __nv_bfloat16>(d, limit);
+  else if (S.fp32) (rc = allow_smem<float, float, float>(d, limit)) || (rc = allow_smem<float, double, float>(d, limit));
+  else rc = allow_smem<double, double, double>(d, limit);
+  if (rc) return rc;
+  q.table_bytes = ((wide ? max_steps : max_table) + 127) / 128 * 128;
   const int dg = d == 7 ? 4 : S.fp32 ? 2 : 1;  // the wider group
   // right-hand sides are staged in the vectors' type; a batch on FP32 factors stages FP64 (one level only)
   const size_t per_cell = std::max(fw[0], bw[0]) + (size_t)dg * (s->pc.levels == 1 && !S.bf16 ? 8 : es);
   const size_t loc = (size_t)dg * max_nc * es;
-  q.ch_log = chunk_log(d == 7 ? FV_VTBE : FV_PPBE);
-  q.smem = 256 + q.table_bytes + (size_t)2 * q.T * dg * es + ((size_t)SLOTS << q.ch_log) * per_cell;
-  if (((SLOTS - 2) << q.ch_log) < widest || q.smem > (size_t)limit) return FV_OK;
-  // the forward result stays in shared memory where that costs no CTA an SM would otherwise hold
-  const int tasks = (q.groups * S.count + sms - 1) / sms, sm_bytes = limit + 1024;
-  const int fit = std::min(sm_bytes / (int)(q.smem + 1024), d == 7 && !S.fp32 ? 1 : std::max(2, 1024 / (q.T + PRODUCERS)));
-  q.loc_smem = !q.wide && q.smem + loc <= (size_t)limit && sm_bytes / (int)(q.smem + loc + 1024) >= std::min(tasks, fit);
-  if (q.loc_smem) q.smem += loc;
+  const int kind = d == 7 ? FV_VTBE : FV_PPBE, tasks = q.groups * S.count, sm_bytes = limit + 1024;
+  const bool heavy = d == 7 && !S.fp32;
+  auto ring_smem = [&](bool small) {
+    return 256 + q.table_bytes + (size_t)2 * q.T * dg * es + ((size_t)1 << (slots_log(kind, small) + chunk_log(kind, small))) * per_cell;
+  };
+  auto held = [&](int var, size_t smem) {  // CTAs an SM holds
+    int n = 0;
+    const void* f = S.bf16 ? kernel_of<float, float, __nv_bfloat16>(d, var) : S.fp32 ? kernel_of<float, float, float>(d, var)
+                                                                                     : kernel_of<double, double, double>(d, var);
+    return smem <= (size_t)limit && !cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, q.T + PRODUCERS, smem) ? n : 0;
+  };
+  // Boxes too many to run at once: a small ring lets an SM hold more of them, where it still holds some steps ahead.
+  // us, large ring (one CTA an SM for FP64 VTBE, three for PPBE), small: FP64 VTBE 3072 boxes of 6^3 cells 2053, 567, of
+  // 10^3 3547, 1391; FP32 VTBE 417, 136 and 786, 337; FP64 PPBE 1296 boxes of 4^3 76, 47; FP32 30, 20
+  const bool small = !wide && widest <= SMALL_STEP && window <= 2 * SMALL_STEP && (long long)sms * held(GLOBAL_LOC, ring_smem(false)) < tasks;
+  q.ch_log = chunk_log(kind, small);
+  q.smem = ring_smem(small);
+  if ((((1 << slots_log(kind, small)) - 2) << q.ch_log) < widest || q.smem > (size_t)limit) return FV_OK;
   const long long CH = 1LL << q.ch_log;
   std::vector<long long> so(S.count + 1, 0);
   for (int b = 0; b < S.count; ++b) so[b + 1] = so[b] + (cell_off[b + 1] - cell_off[b] + CH - 1) / CH * CH;
   q.sT = so[S.count];
+  // Thousands of boxes of a few cells would be padding for the most part (a box is at least a chunk): general sweeps.  Two
+  // by two by two cells are the turn: 24,576 such boxes, general against streamed, FP64 VTBE 781, 1109; FP32 VTBE 296,
+  // 256; FP64 PPBE 166, 190; FP32 PPBE 76, 82 us
+  if (small && q.sT >= (heavy ? 4 : 5) * S.total_cells) return FV_OK;
+  // the forward result stays in shared memory where that costs no CTA an SM would otherwise hold
+  const int per_sm = (tasks + sms - 1) / sms;
+  const int fit = small ? held(SMALL_GLOBAL_LOC, q.smem) : std::min(sm_bytes / (int)(q.smem + 1024), heavy ? 1 : std::max(2, 1024 / (q.T + PRODUCERS)));
+  const bool shared_loc = !wide && q.smem + loc <= (size_t)limit && sm_bytes / (int)(q.smem + loc + 1024) >= std::min(per_sm, fit);
+  if (shared_loc) q.smem += loc;
+  q.variant = wide ? WIDE_ROWS : small ? (shared_loc ? SMALL_SHARED_LOC : SMALL_GLOBAL_LOC) : shared_loc ? SHARED_LOC : GLOBAL_LOC;
   int* ranks = nullptr;
   auto get = [&](void** p, size_t bytes) {
     if (cudaMalloc(p, std::max<size_t>(bytes, 16)) != cudaSuccess) return false;
@@ -775,11 +812,6 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   else pack(0.0);
   FV_CUDA(cudaGetLastError());
   FV_CUDA(cudaDeviceSynchronize());
-  fv_status rc;
-  if (S.bf16) rc = allow_smem<float, float, __nv_bfloat16>(d, limit);
-  else if (S.fp32) (rc = allow_smem<float, float, float>(d, limit)) || (rc = allow_smem<float, double, float>(d, limit));
-  else rc = allow_smem<double, double, double>(d, limit);
-  if (rc) return rc;
   *used = 1;
   return FV_OK;
 }
