@@ -36,7 +36,6 @@ namespace fv {
 namespace {
 
 constexpr int MAX_ROWS = 384;        // cells of the widest step a CTA takes (threads of the solve)
-constexpr int NEAR_TABLE = 48 << 10; // largest step and row tables kept in shared memory (WIDE: the steps alone)
 constexpr int PRODUCERS = 64;        // one warp for the operands, one for the right-hand side
 constexpr unsigned WAIT_TRIES = 1u << 22;
 
@@ -652,7 +651,7 @@ fv_status allow_smem(int d, int limit) {
 // Builds the streams of s when every box fits the scheme: its widest step has a thread for every cell (MAX_ROWS), and
 // an operand ring that holds a whole step fits in shared memory.  *used = 0: the caller keeps the general sweeps,
 // 1.2 to 5 times slower where both can run (us, general against these: PPBE FP32 boxes of 36x36x21 cells 357, 156,
-// 48x48x16 516, 205, 4x96x96 1689, 423; VTBE FP32 24x24x32 1067, 322; VTBE FP64 24x24x32 1736, 596).  Rows are held one
+// 48x48x16 516, 205, 4x96x96 1689, 276; VTBE FP32 24x24x32 1067, 322; VTBE FP64 24x24x32 1736, 596).  Rows are held one
 // step before they begin where MAX_ROWS threads cover such a window (to 36x36x20 cells: a window of 384); the boxes above
 // have steps of 376 to 384 cells and windows to 396, or more rows than shared memory holds a table of, and run WIDE.
 fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::vector<long long>& cell_off, int* used) {
@@ -706,7 +705,6 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   }
   if (widest > MAX_ROWS) return FV_OK;
   q.T = (std::min(window, MAX_ROWS) + 31) / 32 * 32;
-  const bool wide = window > MAX_ROWS || max_table > NEAR_TABLE;
   for (size_t m = 0; m < shapes.size(); ++m) {
     const Shape& sh = shapes[m];
     const int ny = boxes[m][1], nz = boxes[m][2];
@@ -732,7 +730,6 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   else if (S.fp32) (rc = allow_smem<float, float, float>(d, limit)) || (rc = allow_smem<float, double, float>(d, limit));
   else rc = allow_smem<double, double, double>(d, limit);
   if (rc) return rc;
-  q.table_bytes = ((wide ? max_steps : max_table) + 127) / 128 * 128;
   const int dg = d == 7 ? 4 : S.fp32 ? 2 : 1;  // the wider group
   // right-hand sides are staged in the vectors' type; a batch on FP32 factors stages FP64 (one level only)
   const size_t per_cell = std::max(fw[0], bw[0]) + (size_t)dg * (s->pc.levels == 1 && !S.bf16 ? 8 : es);
@@ -748,6 +745,13 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
                                                                                      : kernel_of<double, double, double>(d, var);
     return smem <= (size_t)limit && !cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, q.T + PRODUCERS, smem) ? n : 0;
   };
+  q.table_bytes = (max_table + 127) / 128 * 128;
+  // A row table above 48 KB is read from global memory where it does not fit or would keep out a CTA that has a task (a row
+  // change then waits for its warp's last look ahead: PPBE boxes of 4x96x96 cells, FP32, 144 tasks, 418 us so and 276
+  // from shared memory; FP64, 288 tasks, 617 and 767)
+  const bool wide = window > MAX_ROWS || ring_smem(false) > (size_t)limit ||
+                    (max_table > (48 << 10) && (long long)sms * held(GLOBAL_LOC, ring_smem(false)) < tasks);
+  if (wide) q.table_bytes = (max_steps + 127) / 128 * 128;
   // Boxes too many to run at once: a small ring lets an SM hold more of them, where it still holds some steps ahead.
   // us, large ring (one CTA an SM for FP64 VTBE, three for PPBE), small: FP64 VTBE 3072 boxes of 6^3 cells 2053, 567, of
   // 10^3 3547, 1391; FP32 VTBE 417, 136 and 786, 337; FP64 PPBE 1296 boxes of 4^3 76, 47; FP32 30, 20
