@@ -24,11 +24,13 @@ static void free_system(fv_system* s) {
   free_krylov(s->kry);
   free_batch(s->batch);
   for (void* p : s->allocs) cudaFree(p);
-  if (s->subs.st.err) cudaFreeHost(s->subs.st.err);
+  if (s->words_own) cudaFreeHost(s->words);
   delete s;
 }
 
-static fv_status make_system(const fv_grid* g, int kind, const fv_phys* ph, const fv_pc_desc* pc, fv_system** out) {
+// finer: the system of the finer level, null for the top one
+static fv_status make_system(const fv_grid* g, int kind, const fv_phys* ph, const fv_pc_desc* pc, const fv_system* finer,
+                             fv_system** out) {
   if (pc->inner_gs_passes < 0 || pc->inner_gs_passes > 2)
     return set_error("fv_assemble_system: inner_gs_passes must be 0, 1 or 2"), FV_EINVAL;
   if (pc->levels < 1 || pc->levels > 6) return set_error("fv_assemble_system: levels must be 1..6"), FV_EINVAL;
@@ -42,9 +44,24 @@ static fv_status make_system(const fv_grid* g, int kind, const fv_phys* ph, cons
   s->phys = *ph, s->pc = *pc;
   s->prec32 = pc->precision != FV_PREC_FP64;
   fv_status rc = FV_OK;
+  if (finer) {
+    s->words = finer->words + WORDS, s->words_dev = finer->words_dev + WORDS;
+  } else {
+    const size_t bytes = pc->levels * WORDS * sizeof(int);
+    if (cudaHostAlloc((void**)&s->words, bytes, cudaHostAllocMapped) != cudaSuccess) {
+      delete s;
+      return set_error("fv_assemble_system: allocation of the status words failed"), FV_ENOMEM;
+    }
+    s->words_own = 1;
+    std::memset(s->words, 0, bytes);
+    if (cudaError_t e = cudaHostGetDevicePointer((void**)&s->words_dev, s->words, 0)) {
+      free_system(s);
+      return cuda_fail(e, "fv_assemble_system: status words");
+    }
+  }
   const size_t ng = (size_t)s->d * 6 * 4 * g->h.Nr * (g->h.Ns + 2);
   if (cudaMalloc(&s->ghost, ng * sizeof(double)) != cudaSuccess) {
-    delete s;
+    free_system(s);
     return set_error("fv_assemble_system: ghost layer allocation failed"), FV_ENOMEM;
   }
   s->allocs.push_back(s->ghost);
@@ -99,7 +116,7 @@ static fv_status make_system(const fv_grid* g, int kind, const fv_phys* ph, cons
       }
       cpc.boxes = cboxes.data();
     }
-    if ((rc = make_system(gm->coarse, kind, ph, &cpc, &s->coarse))) {
+    if ((rc = make_system(gm->coarse, kind, ph, &cpc, s, &s->coarse))) {
       free_system(s);
       return rc;
     }
@@ -153,7 +170,7 @@ fv_status fv_assemble_system(const fv_grid* g, int kind, const fv_phys* phys, co
     return set_error("fv_assemble_system: bad argument"), FV_EINVAL;
   if (!(phys->dt > 0) || !(phys->E > 0) || !(phys->Pr > 0) || !(phys->Pm > 0))
     return set_error("fv_assemble_system: E, Pr, Pm, dt must be positive"), FV_EINVAL;
-  return make_system(g, kind, phys, pc, out);
+  return make_system(g, kind, phys, pc, nullptr, out);
 }
 
 fv_status fv_free_system(fv_system* s) {

@@ -105,8 +105,10 @@ struct SweepStream {
   unsigned long long* rows = nullptr;
   int groups = 0, T = 0, ch_log = 0, variant = 0, table_bytes = 0;  // T: threads of the solve; cells a chunk (log2)
   size_t smem = 0;
-  int *err = nullptr, *err_dev = nullptr;  // mapped host word: a wait of the sweep ran out
 };
+
+// words of a system by which its kernels report a wait that ran out
+enum { WORD_SWEEP, WORD_GS64, WORD_GS32, WORDS };
 
 // structured ILU(0) subdomain set of one system on one grid level
 struct Subdomains {
@@ -184,6 +186,9 @@ struct fv_system {
   cudaGraphExec_t inner_graph = nullptr;  // captured inner solve (r32 -> x32)
   int inner_warm = 0;
   unsigned long long inner_buffers = 0;   // fv::inner_buffers() when inner_graph was captured
+  // mapped host memory, one block for a system and its coarse levels (an allocation costs as much as a small assembly)
+  int *words = nullptr, *words_dev = nullptr;  // [WORDS] of this level
+  int words_own = 0;                           // 1: the block begins here and is freed with this system
   unsigned wait_limit = 1u << 24;  // tries after which a wait between blocks gives up
   // FGMRES workspace for this system (outer) sized lazily
   fv::Krylov* kry = nullptr;

@@ -53,7 +53,7 @@ struct KrylovT {
   ArnoldiDev* ad = nullptr; // device-driven solves
   unsigned* ticket = nullptr; // last-block counter of the fused reductions (returns to 0 after each use)
   unsigned* bar = nullptr;    // [3] grid barrier of the one-launch Gram-Schmidt step: arrivals, generation, ran out
-  int *err = nullptr, *err_dev = nullptr;  // mapped host word: a grid barrier ran out
+  int* err = nullptr;         // the system's word (device address): a grid barrier ran out
   unsigned spins = 0;         // bound of a barrier's wait
   int sms = 0, smem = 0;
 };
@@ -75,7 +75,7 @@ unsigned long long inner_buffers(const fv_system* s) {
 template <class T>
 static void free_kt(KrylovT<T>& k) {
   cudaFree(k.V), cudaFree(k.Z), cudaFree(k.w), cudaFree(k.r), cudaFree(k.part), cudaFree(k.h), cudaFree(k.ad), cudaFree(k.ticket), cudaFree(k.bar);
-  cudaFreeHost(k.hhost), cudaFreeHost(k.err);
+  cudaFreeHost(k.hhost);
   k = KrylovT<T>();
 }
 
@@ -115,29 +115,28 @@ static fv_status ensure_krylov(const fv_system* s, int m) {
       cudaMalloc(&k.ad, sizeof(ArnoldiDev)) != cudaSuccess || cudaMalloc(&k.ticket, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(k.ticket, 0, sizeof(unsigned)) != cudaSuccess ||
       cudaMalloc(&k.bar, 3 * sizeof(unsigned)) != cudaSuccess || cudaMemset(k.bar, 0, 3 * sizeof(unsigned)) != cudaSuccess ||
-      cudaHostAlloc((void**)&k.err, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
-      cudaHostGetDevicePointer((void**)&k.err_dev, k.err, 0) != cudaSuccess ||
       cudaMallocHost(&k.hhost, 3 * KMAX * sizeof(double)) != cudaSuccess) {
     free_kt(k);
     return set_error("fv_gmres_solve: device allocation of the Krylov basis failed"), FV_ENOMEM;
   }
-  *k.err = 0;
+  k.err = s->words_dev + (sizeof(T) == 4 ? WORD_GS32 : WORD_GS64);
   return gs_limits<T>(k);
 }
 
 // Whether a grid barrier of s's workspaces (either type) or of its coarse levels' ran out, in work on st, since the last
 // call.  The words are cleared and the barriers made usable again.
 static fv_status gs_failed(const fv_system* s, cudaStream_t st, bool* bad) {
-  auto check = [&](auto& k) -> fv_status {
-    if (!k.err || !*(volatile int*)k.err) return FV_OK;
-    *bad = true, *k.err = 0;
+  auto check = [&](auto& k, int word) -> fv_status {
+    if (!*(volatile int*)(s->words + word)) return FV_OK;
+    *bad = true, s->words[word] = 0;
+    if (!k.bar) return FV_OK;
     FV_CUDA(cudaMemsetAsync(k.bar, 0, 3 * sizeof(unsigned), st));
     FV_CUDA(cudaStreamSynchronize(st));
     return FV_OK;
   };
   fv_status rc;
   for (; s; s = s->coarse)
-    if (s->kry && ((rc = check(s->kry->d)) || (rc = check(s->kry->f)))) return rc;
+    if (s->kry && ((rc = check(s->kry->d, WORD_GS64)) || (rc = check(s->kry->f, WORD_GS32)))) return rc;
   return FV_OK;
 }
 
@@ -857,7 +856,7 @@ static fv_status gs_step(const KrylovT<T>& k, int nv, long long n, const T* w, T
     a.keep = nv > 0 && n % Vec16<T>::L == 0 && smem + keep <= (size_t)k.smem;
     if (a.keep) smem += keep;
     a.n = n, a.passes = nv > 0 ? passes : 0, a.start = nv == 0, a.last = last, a.gj = nv - 1;
-    a.part = k.part, a.h = k.h, a.ad = ad, a.bar = k.bar, a.err = k.err_dev, a.spins = k.spins;
+    a.part = k.part, a.h = k.h, a.ad = ad, a.bar = k.bar, a.err = k.err, a.spins = k.spins;
     const T* V = nv > 0 ? k.V : w;
     void* args[] = {&a, &V, &w, &vout};
     FV_CUDA(cudaLaunchCooperativeKernel(gs_kernel_of<T>(nv, std::make_integer_sequence<int, KMAX>{}), dim3(blocks),

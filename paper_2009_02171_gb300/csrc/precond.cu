@@ -377,10 +377,8 @@ fv_status prepare_sweeps(fv_system* s, int prec) {
   // boxes whose wavefronts fit a CTA run the streamed sweeps (sweep.cu); wider ones the general sweeps below
   if (fv_status rc = build_stream(s, dims, cell_off, &S.st.on)) return rc;
   if (S.st.on) {
-    for (void* p : {(void*)S.off, (void*)S.diag, (void*)S.perm, (void*)S.order, (void*)S.gmap, (void*)S.owned,
-                    (void*)S.gmap_p, (void*)S.owned_p})
-      release(s, p);
-    S.off = S.diag = nullptr, S.perm = S.order = nullptr, S.gmap = S.gmap_p = nullptr, S.owned = S.owned_p = nullptr;
+    release(s, S.off), release(s, S.diag), release(s, S.perm);  // the large ones: giving one back waits for the device
+    S.off = S.diag = nullptr, S.perm = nullptr;
     return FV_OK;
   }
   S.F = S.bf16 ? (void*)dalloc<__nv_bfloat16>(s, (size_t)S.total_cells * Q)

@@ -26,8 +26,10 @@
 #include <algorithm>
 #include <array>
 #include <cstdint>
+#include <cstring>
 #include <map>
 #include <type_traits>
+#include <utility>
 
 #include "fv_internal.h"
 
@@ -632,17 +634,10 @@ fv_status launch(const fv_system* s, int nrhs, const V* r, long long rs, V* z, l
   const Subdomains& S = s->subs;
   const SweepStream& q = S.st;
   SweepArgs a{(const Shape*)q.shapes, q.shape_of, (const int2*)q.steps, q.rows, S.lpt, q.soff, {q.fw[0], q.fw[1]},
-              {q.bw[0], q.bw[1]}, q.gather, loc, q.err_dev, q.sT, s->grid->h.N, rs, zs, S.count, q.T, q.table_bytes};
+              {q.bw[0], q.bw[1]}, q.gather, loc, s->words_dev + WORD_SWEEP, q.sT, s->grid->h.N, rs, zs, S.count, q.T, q.table_bytes};
   void* args[] = {&a, &r, &z};
   FV_CUDA(cudaLaunchKernel(stream_kernel<T, V, FT, KIND>(q.variant), dim3(q.groups * S.count, nrhs), dim3(q.T + PRODUCERS), args,
                            q.smem, st));
-  return FV_OK;
-}
-
-template <class T, class V, class FT>
-fv_status allow_smem(int d, int limit) {
-  for (int var = 0; var < VARIANTS; ++var)
-    FV_CUDA(cudaFuncSetAttribute(kernel_of<T, V, FT>(d, var), cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   return FV_OK;
 }
 
@@ -725,11 +720,6 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   FV_CUDA(cudaGetDevice(&dev));
   FV_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  fv_status rc;
-  if (S.bf16) rc = allow_smem<float, float, __nv_bfloat16>(d, limit);
-  else if (S.fp32) (rc = allow_smem<float, float, float>(d, limit)) || (rc = allow_smem<float, double, float>(d, limit));
-  else rc = allow_smem<double, double, double>(d, limit);
-  if (rc) return rc;
   const int dg = d == 7 ? 4 : S.fp32 ? 2 : 1;  // the wider group
   // right-hand sides are staged in the vectors' type; a batch on FP32 factors stages FP64 (one level only)
   const size_t per_cell = std::max(fw[0], bw[0]) + (size_t)dg * (s->pc.levels == 1 && !S.bf16 ? 8 : es);
@@ -739,11 +729,23 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   auto ring_smem = [&](bool small) {
     return 256 + q.table_bytes + (size_t)2 * q.T * dg * es + ((size_t)1 << (slots_log(kind, small) + chunk_log(kind, small))) * per_cell;
   };
+  // kernels of a variant (FP32 factors: right-hand sides in FP32 and, in a batch, FP64)
+  auto kernels = [&](int var) -> std::array<const void*, 2> {
+    if (S.bf16) return {kernel_of<float, float, __nv_bfloat16>(d, var), nullptr};
+    if (S.fp32) return {kernel_of<float, float, float>(d, var), kernel_of<float, double, float>(d, var)};
+    return {kernel_of<double, double, double>(d, var), nullptr};
+  };
+  auto allow = [&](int var) {
+    for (const void* f : kernels(var))
+      if (f && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) return false;
+    return true;
+  };
   auto held = [&](int var, size_t smem) {  // CTAs an SM holds
     int n = 0;
-    const void* f = S.bf16 ? kernel_of<float, float, __nv_bfloat16>(d, var) : S.fp32 ? kernel_of<float, float, float>(d, var)
-                                                                                     : kernel_of<double, double, double>(d, var);
-    return smem <= (size_t)limit && !cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, q.T + PRODUCERS, smem) ? n : 0;
+    return smem <= (size_t)limit && allow(var) &&
+                   !cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernels(var)[0], q.T + PRODUCERS, smem)
+               ? n
+               : 0;
   };
   q.table_bytes = (max_table + 127) / 128 * 128;
   // A row table above 48 KB is read from global memory where it does not fit or would keep out a CTA that has a task (a row
@@ -773,37 +775,36 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   const bool shared_loc = !wide && q.smem + loc <= (size_t)limit && sm_bytes / (int)(q.smem + loc + 1024) >= std::min(per_sm, fit);
   if (shared_loc) q.smem += loc;
   q.variant = wide ? WIDE_ROWS : small ? (shared_loc ? SMALL_SHARED_LOC : SMALL_GLOBAL_LOC) : shared_loc ? SHARED_LOC : GLOBAL_LOC;
-  int* ranks = nullptr;
-  auto get = [&](void** p, size_t bytes) {
-    if (cudaMalloc(p, std::max<size_t>(bytes, 16)) != cudaSuccess) return false;
-    s->allocs.push_back(*p);
-    return true;
+  if (!allow(q.variant)) return cuda_fail(cudaGetLastError(), "fv_assemble_system: shared memory of the sweeps");
+  // one allocation for the tables (one copy), one for the streams, the cell map and the forward results
+  size_t at = 0;
+  auto part = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 255) / 256 * 256;
+    return o;
   };
-  if (!get((void**)&q.soff, so.size() * sizeof(long long)) || !get((void**)&q.fw[0], fw[0] * q.sT) ||
-      !get((void**)&q.fw[1], fw[1] * q.sT) || !get((void**)&q.bw[0], bw[0] * q.sT) ||
-      !get((void**)&q.bw[1], bw[1] * q.sT) || !get((void**)&q.gather, q.sT * sizeof(int)) || !get((void**)&q.loc, (size_t)d * q.sT * es) ||
-      !get(&q.shapes, shapes.size() * sizeof(Shape)) || !get((void**)&q.shape_of, shape_of.size() * sizeof(int)) ||
-      !get(&q.steps, steps.size() * sizeof(int2)) || !get((void**)&q.rows, rows.size() * sizeof(unsigned long long)) ||
-      !get((void**)&ranks, rank_of.size() * sizeof(int)))
-    return set_error("fv_assemble_system: allocation of sweep data failed"), FV_ENOMEM;
-  if (!q.err) {
-    FV_CUDA(cudaHostAlloc((void**)&q.err, sizeof(int), cudaHostAllocMapped));
-    *q.err = 0;
-    FV_CUDA(cudaHostGetDevicePointer((void**)&q.err_dev, q.err, 0));
+  const size_t t_soff = part(so.size() * sizeof(long long)), t_shapes = part(shapes.size() * sizeof(Shape)),
+               t_steps = part(steps.size() * sizeof(int2)), t_rows = part(rows.size() * sizeof(unsigned long long)),
+               t_of = part(shape_of.size() * sizeof(int)), t_ranks = part(rank_of.size() * sizeof(int)), tables = at;
+  at = 0;
+  const size_t b_fw[2] = {part(fw[0] * q.sT), part(fw[1] * q.sT)}, b_bw[2] = {part(bw[0] * q.sT), part(bw[1] * q.sT)},
+               b_loc = part((size_t)d * q.sT * es), b_gather = part(q.sT * sizeof(int)), bytes = at;
+  unsigned char *tab = nullptr, *str = nullptr;
+  for (auto [p, n] : {std::pair{&tab, tables}, std::pair{&str, bytes}}) {
+    if (cudaMalloc(p, n) != cudaSuccess) return set_error("fv_assemble_system: allocation of sweep data failed"), FV_ENOMEM;
+    s->allocs.push_back(*p);
   }
-  auto put = [](void* to, const void* from, size_t bytes) { return cudaMemcpy(to, from, bytes, cudaMemcpyHostToDevice); };
-  FV_CUDA(put(q.soff, so.data(), so.size() * sizeof(long long)));
-  FV_CUDA(put(q.shapes, shapes.data(), shapes.size() * sizeof(Shape)));
-  FV_CUDA(put(q.shape_of, shape_of.data(), shape_of.size() * sizeof(int)));
-  FV_CUDA(put(q.steps, steps.data(), steps.size() * sizeof(int2)));
-  FV_CUDA(put(q.rows, rows.data(), rows.size() * sizeof(unsigned long long)));
-  FV_CUDA(put(ranks, rank_of.data(), rank_of.size() * sizeof(int)));
+  std::vector<unsigned char> host(tables);
+  auto put = [&](size_t o, const auto& v) { std::memcpy(host.data() + o, v.data(), v.size() * sizeof(v[0])); };
+  put(t_soff, so), put(t_shapes, shapes), put(t_steps, steps), put(t_rows, rows), put(t_of, shape_of), put(t_ranks, rank_of);
+  FV_CUDA(cudaMemcpy(tab, host.data(), tables, cudaMemcpyHostToDevice));
+  q.soff = (long long*)(tab + t_soff), q.shapes = tab + t_shapes, q.steps = tab + t_steps, q.shape_of = (int*)(tab + t_of);
+  q.rows = (unsigned long long*)(tab + t_rows);
+  const int* ranks = (const int*)(tab + t_ranks);
+  for (int g = 0; g < 2; ++g) q.fw[g] = str + b_fw[g], q.bw[g] = str + b_bw[g];
+  q.loc = str + b_loc, q.gather = (int*)(str + b_gather);
+  FV_CUDA(cudaMemset(str, 0, b_gather));  // factors, and padding cells of the forward results: copied, never used
   FV_CUDA(cudaMemset(q.gather, 0xff, q.sT * sizeof(int)));  // padding cells gather nothing
-  FV_CUDA(cudaMemset(q.loc, 0, (size_t)d * q.sT * es));  // padding cells are copied, never used
-  for (int g = 0; g < 2; ++g) {
-    FV_CUDA(cudaMemset(q.fw[g], 0, fw[g] * q.sT));
-    FV_CUDA(cudaMemset(q.bw[g], 0, bw[g] * q.sT));
-  }
   const int blocks = (int)std::min<long long>((S.total_cells + 127) / 128, 152LL * 64);
   auto pack = [&](auto zero) {
     using FT = decltype(zero);
@@ -840,7 +841,7 @@ fv_status ras_stream64(const fv_system* s, int nrhs, const double* r, long long 
 bool sweep_failed(const fv_system* s) {
   bool bad = false;
   for (; s; s = s->coarse)
-    if (s->subs.st.err && *(volatile int*)s->subs.st.err) bad = true, *s->subs.st.err = 0;
+    if (*(volatile int*)(s->words + WORD_SWEEP)) bad = true, s->words[WORD_SWEEP] = 0;
   return bad;
 }
 
