@@ -154,3 +154,26 @@ def test_adam_two_steps_worked_example():
     assert np.allclose(w, [-0.1])
     w, m, v = unet.adam_step(w, np.array([-3.0]), m, v, 2, 0.1, 0.5, 0.75, 0.0)
     assert np.allclose(w, [-0.1 - 0.1 * (-1.25 / 0.75) / np.sqrt(2.4375 / 0.4375)])
+
+
+@pytest.mark.parametrize('layer', ['e0a', 'e0b', 'out'])
+def test_gradients_without_a_coarser_level_match_finite_differences(layer):
+    rng = np.random.default_rng(6)
+    params = {k: (0.3 * rng.standard_normal((co, ci, 3, 3, 3)), 0.1 * rng.standard_normal(co))
+              for k, (ci, co) in unet.layer_shapes(4, 0).items()}
+    r = rng.standard_normal((12, 2, 3, 4, 4))
+    e = rng.standard_normal((12, 2, 3, 4, 4))
+    _, grads = unet.loss_and_grads(params, r, e, 0)
+    w, b = params[layer]
+    h = 1e-6
+    for idx in [(0, 0, 1, 1, 1), (w.shape[0] - 1, w.shape[1] - 1, 0, 2, 1), (1, 0, 2, 0, 2)]:
+        d = np.zeros_like(w)
+        d[idx] = h
+        fd = (unet.loss_and_grads(dict(params, **{layer: (w + d, b)}), r, e, 0)[0] -
+              unet.loss_and_grads(dict(params, **{layer: (w - d, b)}), r, e, 0)[0]) / (2 * h)
+        assert abs(fd - grads[layer][0][idx]) < 1e-6 * max(1.0, abs(fd)), (layer, idx, fd, grads[layer][0][idx])
+    d = np.zeros_like(b)
+    d[-1] = h
+    fd = (unet.loss_and_grads(dict(params, **{layer: (w, b + d)}), r, e, 0)[0] -
+          unet.loss_and_grads(dict(params, **{layer: (w, b - d)}), r, e, 0)[0]) / (2 * h)
+    assert abs(fd - grads[layer][1][-1]) < 1e-6 * max(1.0, abs(fd))
