@@ -25,9 +25,8 @@ struct Field {
 };
 
 // one-sided face mean of component c on panel p.  type 0: xi face f = i
-// (cells i-1, i of row j); type 1: eta face f = j (rows j-1, j of column i);
-// type 2: radial face kf = k (levels k-1, k).  General form: either cell may be a
-// panel-edge ghost or a wall ghost.
+// (cells i-1, i of row j); type 1: eta face f = j (rows j-1, j of column i), either
+// cell a panel-edge ghost perhaps; type 2: the radial face of a wall, k = 0 or Nr.
 __device__ __noinline__ double face_val_any(const Geo& G, const Field& F, int c, int p, int type, int k, int j, int i) {
   ApplyAcc<double> acc(G, F.x, F.gh);
   if (type == 0) {
@@ -36,9 +35,6 @@ __device__ __noinline__ double face_val_any(const Geo& G, const Field& F, int c,
   } else if (type == 1) {
     emit_h(G, acc, 0.5, p, k, j - 1, i, c);
     emit_h(G, acc, 0.5, p, k, j, i, c);
-  } else if (k > 0 && k < G.Nr) {
-    acc.cell(0.5, p, k - 1, j, i, c);
-    acc.cell(0.5, p, k, j, i, c);
   } else {
     const int kc = k == 0 ? 0 : G.Nr - 1;
     acc.cell(0.5, p, kc, j, i, c);
@@ -47,31 +43,16 @@ __device__ __noinline__ double face_val_any(const Geo& G, const Field& F, int c,
   return acc.sum;
 }
 
-// The same mean when both cells are interior cells of panel p (the common case): two loads,
-// the same arithmetic as the general form (0.5 x1, then fma with 0.5 x2).
-__device__ __forceinline__ double face_val(const Geo& G, const Field& F, int c, int p, int type, int k, int j, int i) {
-  const int Ns = G.Ns;
-  long long d = -1;
-  if (type == 0 && i > 0 && i < Ns) d = 1;
-  else if (type == 1 && j > 0 && j < Ns) d = Ns;
-  else if (type == 2 && k > 0 && k < G.Nr) d = (long long)Ns * Ns;
-  if (d < 0) return face_val_any(G, F, c, p, type, k, j, i);
-  const double* xc = F.x + (long long)c * G.N + ((long long)(p * G.Nr + k) * Ns + j) * Ns + i;
-  return fma(0.5, xc[0], 0.5 * xc[-d]);
-}
-
-// face area vector S_f (Cartesian) of face (type, k, j, i) of panel p: the panel's tabulated vector times
-// the radius factor of the level (r_k for horizontal faces, r_f^2 for radial ones)
+// face area vector S_f (Cartesian) of a horizontal face (type 0 xi, 1 eta; k, j, i) of panel p: the panel's tabulated
+// vector times the level's radius
 __device__ __forceinline__ void face_area(const Geo& G, int p, int type, int k, int j, int i, double S[3]) {
-  const double* l;
-  double sc;
   const int Ns = G.Ns;
-  if (type == 0) l = G.sxp + 3 * (((long long)p * Ns + j) * (Ns + 1) + i), sc = G.rc[k];
-  else if (type == 1) l = G.syp + 3 * (((long long)p * (Ns + 1) + j) * Ns + i), sc = G.rc[k];
-  else l = G.srp + 3 * (((long long)p * Ns + j) * Ns + i), sc = G.rf2[k];
+  const double* l = type == 0 ? G.sxp + 3 * (((long long)p * Ns + j) * (Ns + 1) + i) : G.syp + 3 * (((long long)p * (Ns + 1) + j) * Ns + i);
+  const double sc = G.rc[k];
   S[0] = l[0] * sc, S[1] = l[1] * sc, S[2] = l[2] * sc;
 }
 
+// flux through a panel-edge face
 template <int MODE>
 __device__ __forceinline__ void face_flux(const Geo& G, const Field& F, double cL, int p, int type, int k, int j, int i,
                                        double* out) {
@@ -79,7 +60,7 @@ __device__ __forceinline__ void face_flux(const Geo& G, const Field& F, double c
   face_area(G, p, type, k, j, i, S);
   if (MODE == MODE_NL) {
     double v[7];
-    for (int c = 0; c < 7; ++c) v[c] = face_val(G, F, c, p, type, k, j, i);
+    for (int c = 0; c < 7; ++c) v[c] = face_val_any(G, F, c, p, type, k, j, i);
     const double un = v[0] * S[0] + v[1] * S[1] + v[2] * S[2];
     const double bn = v[4] * S[0] + v[5] * S[1] + v[6] * S[2];
     for (int c = 0; c < 3; ++c) {
@@ -89,11 +70,11 @@ __device__ __forceinline__ void face_flux(const Geo& G, const Field& F, double c
     out[3] = -un * v[3];
   } else if (MODE == MODE_DIV) {
     double u[3], b[3];
-    for (int c = 0; c < 3; ++c) u[c] = face_val(G, F, c, p, type, k, j, i), b[c] = face_val(G, F, 4 + c, p, type, k, j, i);
+    for (int c = 0; c < 3; ++c) u[c] = face_val_any(G, F, c, p, type, k, j, i), b[c] = face_val_any(G, F, 4 + c, p, type, k, j, i);
     out[0] = u[0] * S[0] + u[1] * S[1] + u[2] * S[2];
     out[1] = b[0] * S[0] + b[1] * S[1] + b[2] * S[2];
   } else {
-    const double P = face_val(G, F, 0, p, type, k, j, i), Pb = face_val(G, F, 1, p, type, k, j, i);
+    const double P = face_val_any(G, F, 0, p, type, k, j, i), Pb = face_val_any(G, F, 1, p, type, k, j, i);
     for (int c = 0; c < 3; ++c) out[c] = P * S[c], out[3 + c] = Pb * S[c];
   }
 }

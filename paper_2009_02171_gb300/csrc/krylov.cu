@@ -750,7 +750,7 @@ static fv_status gs_limits(KrylovT<T>& k) {
 }
 
 // Blocks and shared memory of the one-launch step for vectors of n; 0 blocks: the slice does not fit (the separate
-// passes below stream such vectors at HBM rate: FP64 above 3.7M, FP32 above 7.4M elements).  At least 1024 elements
+// passes below stream such vectors at HBM rate: FP64 above 3.5M, FP32 above 7.1M elements).  At least 1024 elements
 // a block: fewer only add partials and arrivals at the barrier.
 template <class T>
 static int gs_blocks(const KrylovT<T>& k, long long n, long long* slice, size_t* smem) {

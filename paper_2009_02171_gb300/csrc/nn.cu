@@ -9,16 +9,16 @@
 // each edge (written by whichever kernel produces the tensor: the convolution epilogue,
 // the input packing, the pooling); ring corners stay zero.  A convolution is an implicit
 // GEMM (M = voxels, N = output channels, K = 27 taps x input channels) on the
-// tensor cores (mma.sync m16n8k16, BF16 x BF16 -> FP32): one CTA computes a
-// 4 x 4 x 8 brick of output voxels from a (6 x 6 x 10)-voxel halo of its input
-// and all 27 taps' weights, both staged in shared memory (row stride padded by 8
+// tensor cores (mma.sync m16n8k16, BF16 x BF16 -> FP32): a CTA keeps all 27 taps'
+// weights in shared memory and walks over 4 x 4 x 8 bricks of output voxels, each
+// from a (6 x 6 x 10)-voxel halo of its input, staged too (row stride padded by 8
 // channels so ldmatrix rows fall in distinct banks).  The backward data pass is the same kernel with flipped,
 // transposed weights over the whole padded plane (the gradient of the ring
 // included), followed by halo_adjoint (ring gradients added to the neighbour
 // cells they were copied from); the weight gradient is a GEMM over voxels
-// (M = input channels, N = output channels) split over (tap, voxel range) CTAs,
-// whose partial tiles are added in a fixed order (no atomics: training is bitwise
-// reproducible).
+// (M = input channels, N = output channels) split over (voxel range, dz, 32 input
+// channels) CTAs, nine taps each, whose partial tiles are added in a fixed order (no
+// atomics: training is bitwise reproducible).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -486,8 +486,10 @@ constexpr int WG_GROUPS = 48;   // voxel-range groups of the weight gradient (pa
 constexpr int BG_BLOCKS = 640;  // blocks of the bias gradient (partial sums)
 constexpr int SS_BLOCKS = 320;  // blocks per sample of the sum of squares
 constexpr int WG_THREADS = 9 * 32;
+constexpr int WG_STAGES = 4;    // chunk buffers: at most 51,920 bytes each (rows of 63 cells, 32 channels)
+constexpr int WG_SMEM = 220 * 1024;
 
-template <int CIN, int GC, int STAGES>
+template <int CIN, int GC>
 __global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const __grid_constant__ WGradArgs a) {
   constexpr int cs = CIN + 8, gsn = GC + 8, MT = CIN / 16, NT2 = GC / 16, qx = CIN / 8, qg = GC / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -552,22 +554,20 @@ __global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const __grid_constant
       at[kk] = (r * 3 + dy) * a.pw + x + dx - (r == 0 ? x00 : 0);
     }
   };
-  // STAGES - 1 chunks ahead, one commit group a chunk; with one buffer a chunk is copied when the last is done
-  constexpr int AHEAD = STAGES > 1 ? STAGES - 1 : 1;
+  // WG_STAGES - 1 chunks ahead, one commit group a chunk
+  constexpr int AHEAD = WG_STAGES - 1;
 #pragma unroll
   for (int u = 0; u < AHEAD; ++u) {
     if (c_begin + u < c_end) stage(c_begin + u, buf + u * STG);
     cp_commit();
   }
   int turn = 0;
-  for (long long ch = c_begin; ch < c_end; ++ch, turn = turn + 1 == STAGES ? 0 : turn + 1) {
+  for (long long ch = c_begin; ch < c_end; ++ch, turn = turn + 1 == WG_STAGES ? 0 : turn + 1) {
     if (ch == c_begin || !fixed || ch + 1 == nchunk) rows_of(ch);
     cp_wait<AHEAD - 1>();
     __syncthreads();  // chunk ch has landed, the buffer of chunk ch - 1 is free
-    if (STAGES > 1) {
-      if (ch + AHEAD < c_end) stage(ch + AHEAD, buf + (turn == 0 ? STAGES - 1 : turn - 1) * STG);
-      cp_commit();
-    }
+    if (ch + AHEAD < c_end) stage(ch + AHEAD, buf + (turn == 0 ? WG_STAGES - 1 : turn - 1) * STG);
+    cp_commit();
     const uint32_t xb = (uint32_t)__cvta_generic_to_shared(buf + turn * STG), gb = xb + (uint32_t)(rows * cs * 2);
 #pragma unroll
     for (int kk = 0; kk < WK / 16; ++kk) {
@@ -585,11 +585,6 @@ __global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const __grid_constant
           mma16816(acc[mt][nt][1], af, bf[nt][2], bf[nt][3]);
         }
       }
-    }
-    if (STAGES == 1) {
-      __syncthreads();
-      if (ch + 1 < c_end) stage(ch + 1, buf);
-      cp_commit();
     }
   }
   const int tap = blockIdx.y * 9 + warp;
@@ -926,29 +921,21 @@ ConvArgs bwd_args(const bf16* g, const NetLayer& ly, bf16* out, int P, const Lvl
   return a;
 }
 
-constexpr int WG_SMEM = 220 * 1024;
-
-template <int CIN, int GC, int STAGES>
-fv_status wgrad_launch_n(const WGradArgs& a, int cin, int groups, size_t stage, cudaStream_t st) {
+template <int CIN, int GC>
+fv_status wgrad_launch(const WGradArgs& a, int cin, int groups, cudaStream_t st) {
+  const size_t smem = WG_STAGES * ((size_t)a.nr * 3 * a.pw * (CIN + 8) + WK * (GC + 8)) * 2;
+  if (smem > (size_t)WG_SMEM) return set_error("fv_net: weight-gradient chunk too large"), FV_EINVAL;
   static std::once_flag once[64];
   static cudaError_t err[64];
   int dev = 0;
   FV_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return set_error("fv_net: device ordinal out of range"), FV_EINVAL;
   std::call_once(once[dev], [&] {
-    err[dev] = cudaFuncSetAttribute(wgrad_kernel<CIN, GC, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
+    err[dev] = cudaFuncSetAttribute(wgrad_kernel<CIN, GC>, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
   });
   FV_CUDA(err[dev]);
-  wgrad_kernel<CIN, GC, STAGES><<<dim3(groups, 3, cin / CIN), WG_THREADS, STAGES * stage, st>>>(a);
+  wgrad_kernel<CIN, GC><<<dim3(groups, 3, cin / CIN), WG_THREADS, smem, st>>>(a);
   return FV_OK;
-}
-
-// four buffers where they fit (rows of 4 cells and more), else one: at most 64 rows of 3 x 3 voxels, 57 KB
-template <int CIN, int GC>
-fv_status wgrad_launch(const WGradArgs& a, int cin, int groups, cudaStream_t st) {
-  const size_t stage = ((size_t)a.nr * 3 * a.pw * (CIN + 8) + WK * (GC + 8)) * 2;
-  return 4 * stage <= (size_t)WG_SMEM ? wgrad_launch_n<CIN, GC, 4>(a, cin, groups, stage, st)
-                                      : wgrad_launch_n<CIN, GC, 1>(a, cin, groups, stage, st);
 }
 
 fv_status wgrad(fv_net* n, const bf16* s0, int c0, const bf16* s1, int c1, const bf16* g, int gc, int li, int P,
