@@ -15,12 +15,14 @@
 // one cp.async two levels ahead, halo cells across a panel edge the quadratic ghost interpolants.  Every x value is
 // read from HBM once (plus the planes at chunk boundaries) and every y value is written once.
 // What bounds it: FP64 its multiply-adds (16 cycles of the SM's FP64 pipe each); FP32 the instructions issued.  So
-// the nine horizontal weights and the radial weight carry 1 / sigma from the start (14 multiply-adds a value and
+// the nine horizontal weights and the radial weight carry 1 / sigma in their tables (14 multiply-adds a value and
 // level), weights, metric and couplings are shared by a group's components in registers, and shared memory is read
 // 16 bytes at a time.  The panel-edge fluxes of a tile are copied beside its planes: as loads behind per-cell tests
 // they were 2/3 of the instructions (every warp of a 64-cell panel has an edge lane).
-// Against one CTA a component with four rows a thread, both launches, us on GB300: FP64 VTBE 6x64^3 640 -> 526 (FP64
-// pipe), PPBE 6x45^2x39 120 -> 62; FP32 VTBE 6x128^2x96 627 -> 360, 6x64^3 134 -> 93, PPBE 6x32^3 25 -> 14.
+// Against one CTA a component with four rows a thread, both launches, us on GB300: FP64 VTBE 6x64^3 640 -> 517 (FP64
+// pipe), PPBE 6x45^2x39 120 -> 62; FP32 VTBE 6x128^2x96 627 -> 353, 6x64^3 134 -> 93, PPBE 6x32^3 25 -> 14.  The tables'
+// products are taken in FP64 and rounded once (as FP32 products here the error against 64 bits was above that of
+// the earlier kernel: PPBE 6x33^2x17 9.1e-8, then 8.6e-8, now 8.4e-8; VTBE 6x128^2x96 5.0e-8, 5.0e-8, 4.8e-8).
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -329,14 +331,12 @@ __device__ __forceinline__ void tile_body(const GT& G, const Coefs<T>& cf, const
       for (int c = 0; c < NG; ++c) sh[(k & (RING - 1)) * SLOT + c * CS + hpos] = hv[c];
   };
   // per-cell constants: weights over sigma, unit radius vector
-  T w[CPT][9], cr[CPT], rh[CPT][3];
+  T w[CPT][9], rh[CPT][3];
 #pragma unroll
   for (int m = 0; m < CPT; ++m) {
     const int ji = act && ig + m < wi ? own + m : 0;
-    const T is = G.invsig[ji];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[m][q] = G.w9[9 * ji + q] * is;
-    cr[m] = G.crf[ji] * is;
+    for (int q = 0; q < 9; ++q) w[m][q] = G.w9[9 * ji + q];
     if constexpr (KIND == FV_VTBE) {
       const T xl[3] = {G.xhat[3 * ji], G.xhat[3 * ji + 1], G.xhat[3 * ji + 2]};
       rotate_exact(p, xl, rh[m]);
@@ -438,7 +438,7 @@ __device__ __forceinline__ void tile_body(const GT& G, const Coefs<T>& cf, const
           if (c < 2) Vals<T>::load(s0 + (1 - c) * CS, uo);
 #pragma unroll
         for (int m = 0; m < CPT; ++m) {
-          const T lap = fma(cr[m], rt * (up[m] - x0[m]) - rb * (x0[m] - dn[m]), h[m]);
+          const T lap = fma(G.crad, rt * (up[m] - x0[m]) - rb * (x0[m] - dn[m]), h[m]);
           T o = KIND == FV_PPBE ? cd * lap : fma(cd, lap, x0[m]);
           if constexpr (UT) {
             if (c < 3) o = fma(c == 0 ? rh[m][0] : c == 1 ? rh[m][1] : rh[m][2], thk[m], o);

@@ -26,6 +26,7 @@ struct GeoT {
   int Ns, Nr;
   long long N;                 // 6 Ns^2 Nr
   R hs, hr, ri, ro;
+  R crad;                      // h_s^2 / h_r    (radial faces, times r_f^2, over sigma)
   R wall_in, wall_out;         // 1 + (r_c/r_g)^2 at the inner / outer wall
   const R* ax11;               // [j][if]  a11 * h_r            (xi faces, Ns x (Ns+1))
   const R* ax12;               // [j][if]  a12 * h_r / 4
@@ -50,8 +51,8 @@ struct GeoT {
   const int* psq;              // [p][side]  its side
   const int* psgn;             // [p][side]  F_p = psgn F_q for the shared face
   const int* ptmap;            // [p][side][t] tangential index on the neighbour side
-  const R* w9;                 // [j][i][9] horizontal 9-point weights of sum_faces F (panel-edge faces left out),
-                               // index (dj + 1) * 3 + (di + 1)
+  const R* w9;                 // [j][i][9] horizontal 9-point weights of sum_faces F over sigma (panel-edge faces
+                               // left out), index (dj + 1) * 3 + (di + 1)
   const GeoT* self;            // device copy of this struct (out-of-line device code reads it
                                // through this pointer so kernels never take a parameter's address)
 };

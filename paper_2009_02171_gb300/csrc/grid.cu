@@ -177,6 +177,7 @@ fv_status build_grid(const fv_grid_desc* desc, fv_grid** out) {
         const double c = ay22[j * Ns + i], e = ay12[j * Ns + i];
         W(0, 0) -= c, W(-1, 0) += c, W(-1, 1) -= e, W(-1, -1) += e, W(0, 1) -= e, W(0, -1) += e;
       }
+      for (int m = 0; m < 9; ++m) w[m] *= invsig[j * Ns + i];  // here, so that the FP32 table is rounded once
     }
 
   // panel-edge ghost interpolation and face pairing, from the geometry
@@ -261,7 +262,7 @@ fv_status build_grid(const fv_grid_desc* desc, fv_grid** out) {
   const std::vector<double> sxp = per_panel(sx), syp = per_panel(sy), srp = per_panel(sr);
 
   Geo& G = g->geo;
-  G.Ns = Ns, G.Nr = Nr, G.N = h.N, G.hs = hs, G.hr = hr, G.ri = h.ri, G.ro = h.ro;
+  G.Ns = Ns, G.Nr = Nr, G.N = h.N, G.hs = hs, G.hr = hr, G.ri = h.ri, G.ro = h.ro, G.crad = hs * hs / hr;
   double rci = h.ri + 0.5 * hr, rgi = h.ri - 0.5 * hr, rco = h.ro - 0.5 * hr, rgo = h.ro + 0.5 * hr;
   G.wall_in = 1.0 + (rci / rgi) * (rci / rgi);
   G.wall_out = 1.0 + (rco / rgo) * (rco / rgo);
@@ -286,7 +287,7 @@ fv_status build_grid(const fv_grid_desc* desc, fv_grid** out) {
   // FP32 copy of the tables for the mixed-precision inner solves
   auto f32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
   GeoF& F = g->geof;
-  F.Ns = Ns, F.Nr = Nr, F.N = h.N, F.hs = (float)hs, F.hr = (float)hr, F.ri = (float)h.ri, F.ro = (float)h.ro;
+  F.Ns = Ns, F.Nr = Nr, F.N = h.N, F.hs = (float)hs, F.hr = (float)hr, F.ri = (float)h.ri, F.ro = (float)h.ro, F.crad = (float)G.crad;
   F.wall_in = (float)G.wall_in, F.wall_out = (float)G.wall_out;
   F.gq = G.gq, F.gsrc = G.gsrc, F.pq = G.pq, F.psq = G.psq, F.psgn = G.psgn, F.ptmap = G.ptmap;
   ok = ok && (F.ax11 = upload(g, f32(ax11))) && (F.ax12 = upload(g, f32(ax12))) && (F.ay22 = upload(g, f32(ay22))) &&
