@@ -76,11 +76,9 @@ def test_fp32_apply_matches_oracle(fv, kind, Ns, Nr):
     fv.fv_free_grid(g)
 
 
-# Sweep variants: VTBE (kind 0) boxes whose widest wavefront step fits the CTA (<= 384 cells) take the
-# register-pipelined level-mapped sweeps.  PPBE boxes of that kind take the shared-memory staged sweeps,
-# 8 steps deep (the small cases) or 4 (40 x 4: 42 x 42 x 4 boxes, 96 threads), or the register-pipelined
-# ones when no 4-deep stage ring fits (32 x 12 with overlap 2: 36 x 36 x 12 boxes, 224 threads, 218 KB).
-# 42 x 42 x 24 (504 cells in a step) takes the level-mapped sweeps with several cells a thread.
+# Boxes whose widest wavefront step has at most 384 cells take the streamed sweeps, with the forward result in shared
+# memory (the small cases) or in global memory (32 x 12 with overlap 2: 36 x 36 x 12 boxes).  42 x 42 x 24 (504 cells in
+# a step) takes the general sweeps with several cells a thread.
 @pytest.mark.parametrize('kind,Ns,Nr,parts,delta', [(0, 8, 6, (2, 2, 2), 1), (1, 10, 8, (3, 2, 2), 2),
                                                      (1, 8, 8, (1, 1, 1), 1), (0, 9, 5, (2, 3, 1), 2),
                                                      (1, 16, 12, (1, 1, 1), 1), (1, 40, 4, (1, 1, 1), 1),
@@ -320,9 +318,9 @@ def test_mixed_precision_three_level_solve_reaches_fp64_residual(fv):
 
 @pytest.mark.parametrize('kind,levels', [(0, 1), (1, 2)])
 def test_bf16_factor_solve_reaches_fp64_residual(fv, kind, levels):
-    """FV_PREC_BF16: the FP32 inner solves read their ILU(0) factors stored in BF16 (every level, staged and
-    register-pipelined sweeps).  The outer FP64 FGMRES still reaches a true FP64 residual of 1e-8 against the
-    oracle's matrix, in at most two more outer iterations than with FP32 factors."""
+    """FV_PREC_BF16: the FP32 inner solves read their ILU(0) factors stored in BF16 (every level).  The outer FP64
+    FGMRES still reaches a true FP64 residual of 1e-8 against the oracle's matrix, in at most two more outer
+    iterations than with FP32 factors."""
     Ns = Nr = 12
     A, d, disc = _oracle_matrix(kind, Ns, Nr)
     b = random_vector(A.shape[0], 23)

@@ -16,10 +16,10 @@ PH = dict(E=1e-3, Ra=100.0, Pr=1.0, Pm=5.0, dt=1e-4)
 @pytest.mark.parametrize('kind,Ns,Nr,parts,delta', [
     (1, 4, 2, (4, 4, 2), 0),      # boxes of one cell
     (0, 5, 3, (2, 2, 3), 1),      # VTBE, one-warp windows, odd boxes
-    (1, 24, 16, (1, 1, 1), 0),    # 6144 cells a box: more chunks than the ring holds, both directions
+    (1, 24, 16, (1, 1, 1), 0),    # 9216 cells a box: more chunks than the ring holds, both directions
     (0, 20, 14, (1, 1, 1), 1),    # VTBE with the forward result in global memory
-    (1, 28, 26, (1, 1, 1), 0),    # a window of 377 rows: 384 threads, the most the streamed sweeps take
-    (1, 28, 32, (1, 1, 1), 0),    # 461 rows: the general sweeps
+    (1, 28, 26, (1, 1, 1), 0),    # a window of 377 rows: 384 threads
+    (1, 28, 32, (1, 1, 1), 0),    # steps of more than 384 cells: the general sweeps
     (1, 11, 7, (3, 2, 2), 2),     # uneven boxes
     (0, 13, 9, (3, 2, 2), 2)])
 def test_sweeps_match_oracle(kind, Ns, Nr, parts, delta):
