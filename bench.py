@@ -66,7 +66,8 @@ METRIC = 'wall time per time step at 1e-8 residual'
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a kernel category at the default
 # workload, from the ncu capture in the file named beside it; a category leaves this table when its kernels
 # change, until they are captured again
-TRAFFIC = {}
+TRAFFIC = {'net_fwd': (49793877, 'profiles/launches_net_forward_c16_coarse32.md'),
+           'apply_vtbe_fp32': (57350656, 'profiles/ncu_apply_vtbe_shell64.md')}
 # CPU oracle: wall-clock budget for its real time steps (after its setup); at least one step always runs
 ORACLE_BUDGET_S = float(os.environ.get('FV_ORACLE_BUDGET_S', '100'))
 

@@ -48,3 +48,7 @@ def test_stable_dt_keeps_the_alfven_cfl_number_below_the_target():
         dt = bench.stable_dt(c)
         assert 0.8 < c * dt <= bench.CFL_TARGET
         assert float('%.2g' % dt) == dt
+
+
+def test_measured_traffic_is_known_for_the_kernels_the_roofline_names():
+    assert {'net_fwd', 'apply_vtbe_fp32'} <= set(bench.TRAFFIC)
