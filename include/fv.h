@@ -208,8 +208,8 @@ fv_status fv_gmres_solve(const fv_system* s, const double* b, double* x, const f
  * The preconditioner is the system's one-level RAS (levels = 1 only), with
  * FP32 subdomain solves when the system was assembled with FV_PREC_FP32,
  * one launch over all (subdomain, right-hand side) pairs.  Subdomains too wide
- * for that (above 384 cells in a wavefront): every factor loaded is
- * applied to a group of right-hand sides (the group size is tuned by timing
+ * for that (above 384 cells in a wavefront), or thousands of a few cells each:
+ * every factor loaded is applied to a group of right-hand sides (the group size is tuned by timing
  * on the first call for a given nrhs), in one persistent launch a direction
  * that takes subdomains largest first.
  * stats: NULL or nrhs entries. */

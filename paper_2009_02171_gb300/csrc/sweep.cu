@@ -16,9 +16,9 @@
 //    are that row's last three values, of which two are already in registers: a step reads two values from a
 //    two-deep ring in shared memory, does two dependent multiply-adds a component, stores one and meets a barrier.
 //  * Operands are streamed.  A cell's factors and its grid cell are packed into 16-byte words, chunk by chunk; one
-//    thread keeps a ring of eight (small: four) chunks filled with cp.async.bulk, ahead of the steps by as much as the ring
-//    holds, and a second warp gathers the right-hand side through the cell map (forward) or reads the forward
-//    result back (backward) with cp.async, completion counted by mbarriers.
+//    thread keeps a ring of chunks filled with cp.async.bulk, ahead of the steps by as much as the ring holds, and a
+//    second warp gathers the right-hand side through the cell map (forward) or reads the forward result back
+//    (backward) with cp.async, completion counted by mbarriers.
 // Positions outside the box have exactly zero factors (assembly writes zero there and the factorization never
 // updates them), so every neighbour is read unconditionally from a ring that starts at zero.
 #include <cuda_bf16.h>
@@ -203,7 +203,7 @@ enum Variant { GLOBAL_LOC, SHARED_LOC, WIDE_ROWS, SMALL_GLOBAL_LOC, SMALL_SHARED
 // chunks of the operand ring (log2), cells a chunk (log2)
 __host__ __device__ constexpr int slots_log(int kind, bool small) { return small && kind == FV_VTBE ? 2 : 3; }
 __host__ __device__ constexpr int chunk_log(int kind, bool small) { return small ? 5 : kind == FV_VTBE ? 6 : 7; }
-constexpr int SMALL_STEP = 64;  // widest step of the small ring: it holds three and more steps ahead of the solve
+constexpr int SMALL_STEP = 64;  // widest step of the small ring, which holds two of them (VTBE) or four (PPBE)
 constexpr int max_threads(int var) { return (var >= SMALL_GLOBAL_LOC ? 2 * SMALL_STEP : MAX_ROWS) + PRODUCERS; }
 constexpr int min_ctas(int var, bool heavy) { return var >= SMALL_GLOBAL_LOC ? (heavy ? 2 : 4) : heavy ? 1 : 2; }
 
@@ -754,7 +754,7 @@ fv_status build_stream(fv_system* s, const std::vector<int>& dims, const std::ve
   const bool wide = window > MAX_ROWS || ring_smem(false) > (size_t)limit ||
                     (max_table > (48 << 10) && (long long)sms * held(GLOBAL_LOC, ring_smem(false)) < tasks);
   if (wide) q.table_bytes = (max_steps + 127) / 128 * 128;
-  // Boxes too many to run at once: a small ring lets an SM hold more of them, where it still holds some steps ahead.
+  // Boxes too many to run at once: a small ring lets an SM hold more of them, where it still holds a step ahead.
   // us, large ring (one CTA an SM for FP64 VTBE, three for PPBE), small: FP64 VTBE 3072 boxes of 6^3 cells 2053, 567, of
   // 10^3 3547, 1391; FP32 VTBE 417, 136 and 786, 337; FP64 PPBE 1296 boxes of 4^3 76, 47; FP32 30, 20
   const bool small = !wide && widest <= SMALL_STEP && window <= 2 * SMALL_STEP && (long long)sms * held(GLOBAL_LOC, ring_smem(false)) < tasks;
